@@ -240,15 +240,19 @@ eat_status run_shared(eat_handle* h, const TcCall& c, const void* x, int T, cuda
     return launch(h, kSDown, ss, "tc shared down",
                   [&] { return tc_launch_down(h->tc, c, true, 1, ss); });
   }
-  const int tpg = (T + kSimtTileRows - 1) / kSimtTileRows;
-  GroupMap gs{nullptr, nullptr, nullptr, kRowIdentity, h->S, T, tpg * h->S};
+  const SimtShape shape = simt_shape(T, h->S, h->Fs);
+  auto groups = [&](int tile_rows) {
+    return GroupMap{nullptr, nullptr, nullptr, kRowIdentity, h->S, T,
+                    (T + tile_rows - 1) / tile_rows * h->S};
+  };
   EAT_TRY(launch(h, kSUp, ss, "shared gate/up", [&] {
-    return launch_ffn_gateup_simt(h->bf16, x, h->desc.ws_gate, h->desc.ws_up, h->Fs, h->d, gs,
-                                  h->sact, ss);
+    return launch_ffn_gateup_simt((const float*)x, (const float*)h->desc.ws_gate,
+                                  (const float*)h->desc.ws_up, h->Fs, h->d,
+                                  groups(simt_rows_up(shape)), shape, (float*)h->sact, ss);
   }));
   return launch(h, kSDown, ss, "shared down", [&] {
-    return launch_ffn_down_simt(h->bf16, h->sact, h->desc.ws_down, h->d, h->Fs, gs,
-                                (float*)h->sout, ss);
+    return launch_ffn_down_simt((const float*)h->sact, (const float*)h->desc.ws_down, h->d, h->Fs,
+                                groups(simt_rows_down(shape)), shape, (float*)h->sout, ss);
   });
 }
 
@@ -267,8 +271,10 @@ bool shared_on_side_stream(const eat_handle* h, int T, int tile_rows) {
 eat_status run_forward(eat_handle* h, const void* x, int T, int ppl_sign, void* y,
                        int32_t* idx_opt, float* w_opt, int32_t* k_opt, cudaStream_t st,
                        const void* x_host = nullptr) {
-  const int tile_rows = h->backend == 1 ? tc_tile_rows(h->tc, T) : kSimtTileRows;
-  const int tile_rows_down = h->backend == 1 ? tc_tile_rows_down(h->tc, T) : kSimtTileRows;
+  const SimtShape shape = simt_shape(T, h->K, h->F);  // (fp32 layers)
+  const int tile_rows = h->backend == 1 ? tc_tile_rows(h->tc, T) : simt_rows_up(shape);
+  const int tile_rows_down =
+      h->backend == 1 ? tc_tile_rows_down(h->tc, T) : simt_rows_down(shape);
   TcCall c;
   c.x = x;
   c.T = T;
@@ -322,14 +328,19 @@ eat_status run_forward(eat_handle* h, const void* x, int T, int ppl_sign, void* 
     EAT_TRY(launch(h, kDown, st, "tc down",
                    [&] { return tc_launch_down(h->tc, c, false, n_split, st); }));
   } else {
-    GroupMap gm{h->perm.offs, h->perm.tile_offs, h->perm.perm_tok, kRowGather, h->E, 0,
-                (rows + kSimtTileRows - 1) / kSimtTileRows + h->E};
+    auto groups = [&](const int32_t* tile_offs, int tr) {
+      return GroupMap{h->perm.offs, tile_offs, h->perm.perm_tok, kRowGather, h->E, 0,
+                      (rows + tr - 1) / tr + std::min(h->E, rows)};
+    };
     EAT_TRY(launch(h, kUp, st, "ffn gate/up", [&] {
-      return launch_ffn_gateup_simt(h->bf16, x, h->desc.w_gate, h->desc.w_up, h->F, h->d, gm,
-                                    h->act, st);
+      return launch_ffn_gateup_simt((const float*)x, (const float*)h->desc.w_gate,
+                                    (const float*)h->desc.w_up, h->F, h->d,
+                                    groups(h->perm.tile_offs, tile_rows), shape, (float*)h->act,
+                                    st);
     }));
     EAT_TRY(launch(h, kDown, st, "ffn down", [&] {
-      return launch_ffn_down_simt(h->bf16, h->act, h->desc.w_down, h->d, h->F, gm, h->opart, st);
+      return launch_ffn_down_simt((const float*)h->act, (const float*)h->desc.w_down, h->d, h->F,
+                                  groups(h->perm.tile_offs2, tile_rows_down), shape, h->opart, st);
     }));
   }
   if (side) {

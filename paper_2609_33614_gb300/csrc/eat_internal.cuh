@@ -149,14 +149,21 @@ struct GroupMap {
   int max_tiles;             // upper bound of the total number of row tiles (grid size)
 };
 
+// fp32 layers run their expert kernels in one of three shapes, chosen by the size of a call of T
+// tokens and K selections (or shared experts) of width F; each shape has its own row tiles.
+enum class SimtShape { kSmall, kMid, kLarge };
+SimtShape simt_shape(int T, int K, int F);
+constexpr int simt_rows_up(SimtShape s) {
+  return s == SimtShape::kLarge ? 64 : s == SimtShape::kMid ? 32 : 16;
+}
+constexpr int simt_rows_down(SimtShape s) { return s == SimtShape::kSmall ? 16 : 32; }
 // act[slot, f] = silu(sum_j in[row, j] Wg[g, f, j]) * (sum_j in[row, j] Wu[g, f, j])
-cudaError_t launch_ffn_gateup_simt(int dtype_bf16, const void* in, const void* wg, const void* wu,
-                                   int Fout, int Kdim, GroupMap gm, void* act, cudaStream_t st);
-// out[slot, c] = sum_f act[slot, f] Wd[g, c, f]   (fp32 output)
-cudaError_t launch_ffn_down_simt(int dtype_bf16, const void* act, const void* wd, int Dout,
-                                 int Kdim, GroupMap gm, float* out, cudaStream_t st);
-constexpr int kSimtTileRows = 32;
-
+cudaError_t launch_ffn_gateup_simt(const float* in, const float* wg, const float* wu, int Fout,
+                                   int Kdim, GroupMap gm, SimtShape shape, float* act,
+                                   cudaStream_t st);
+// out[slot, c] = sum_f act[slot, f] Wd[g, c, f]
+cudaError_t launch_ffn_down_simt(const float* act, const float* wd, int Dout, int Kdim,
+                                 GroupMap gm, SimtShape shape, float* out, cudaStream_t st);
 // ---------------------------------------------------------------------------------------------
 // Combine / unpermute and account update
 // ---------------------------------------------------------------------------------------------

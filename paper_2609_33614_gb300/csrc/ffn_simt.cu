@@ -3,164 +3,310 @@
 // SwiGLU): act = silu(x Wg^T) * (x Wu^T) fused in the first kernel's epilogue; the second kernel
 // is the down projection act Wd^T, written per slot in fp32 for the combine.
 //
-// Tile: 32 rows x 64 output features, K in chunks of 32 staged through shared memory; 256
-// threads, each owning 2 rows x 4 features (x2 for gate and up).  Blocks map to (feature tile,
-// row tile); a row tile belongs to one group (expert), found from the tile prefix.
+// A block computes BR rows x BC weight rows (gate and up rows of BC / 2 features, or BC down
+// features) of one group.  Operands go through shared memory as they lie in memory (K contiguous,
+// cp.async, rows padded by 16 bytes so that eight rows' 16-byte pieces cover all banks); a warp
+// owns a (4 TM) x (8 TN) tile, lane (l / 8, l % 8) the rows l / 8 + 4 i and columns l % 8 + 8 j,
+// and reads TM + TN 16-byte pieces per TM * TN * 4 FMAs.  KG groups of warps take equal shares of
+// each K chunk and their tiles are added through shared memory in group order.
+//
+// What bounds it: a large call the shared-memory reads (8 x 8 outputs per thread need one 16-byte
+// read per 16 FMAs), a small call the latency of one block's tile lookup, copies and sums.  Hence
+// three shapes, by the call's (selected rows) x (expert width); the layer of 8 experts, width 512
+// and d_model 256 measured, us per forward call (small / mid / large shape):
+//   tokens      64    128    384    512    768   1536   1999   3000   4096
+//   small     27.7   34.4   71.4   80.8  106.2  174.8  214.1  303.7  404.2
+//   mid       40.2   46.6   76.2   81.3   93.5  123.5  158.0  203.8  268.7
+//   large     62.1   63.3   91.7  103.8  117.6  146.2  155.6  193.3  266.7
+// (the kernels before, 32 x 64 tiles with 2 x 4 outputs per thread and one chunk in flight: gate/up
+// and down 26.6 + 46.1 us at 64 tokens, 108 + 95 us at 1999.)
 #include "eat_internal.cuh"
+
+#include <mutex>
 
 namespace eat {
 
 namespace {
 
-constexpr int BR = kSimtTileRows;  // rows per tile
-constexpr int BF = 64;             // output features per tile
-constexpr int BK = 32;
-constexpr int kThreads = 256;
-
-__device__ __forceinline__ float ld(const float* p, size_t i) { return p[i]; }
-__device__ __forceinline__ float ld(const __nv_bfloat16* p, size_t i) {
-  return __bfloat162float(p[i]);
-}
-__device__ __forceinline__ void st(float* p, size_t i, float v) { p[i] = v; }
-__device__ __forceinline__ void st(__nv_bfloat16* p, size_t i, float v) {
-  p[i] = __float2bfloat16_rn(v);
-}
-
-struct TileInfo {
-  int g, row0, nrows, slot0;
-  bool ok;
+// BR, BC: rows and weight rows of a block; TM, TN: outputs per thread; KG: warp groups along K;
+// BK: columns of a K chunk; ST: chunks in flight; GATEUP: gate and up rows, or down rows.
+template <bool GATEUP_, int WR_, int WC_, int TM_, int TN_, int KG_, int BK_, int ST_, int MINB_>
+struct SimtCfg {
+  static constexpr bool GATEUP = GATEUP_;
+  static constexpr int WR = WR_, WC = WC_, TM = TM_, TN = TN_, KG = KG_, BK = BK_, ST = ST_;
+  static constexpr int MINB = MINB_;  // blocks an SM should hold (register bound)
+  static constexpr int BR = WR * 4 * TM, BC = WC * 8 * TN;
+  static constexpr int FEAT = GATEUP ? BC / 2 : BC;  // output features of a block
+  static constexpr int THREADS = 32 * WR * WC * KG;
+  static constexpr int LD = BK + 4;  // floats between the rows of a chunk in shared memory
+  static constexpr int STAGE = (BR + BC) * LD;
+  static constexpr int RED = KG > 1 ? KG * BR * (BC + 1) : 0;  // partial tiles (reuse the ring)
+  static constexpr int SMEM = 4 * (ST * STAGE > RED ? ST * STAGE : RED);
+  static_assert(BK % (4 * KG) == 0, "K share of a warp group in 16-byte pieces");
 };
+using SimtLargeUp = SimtCfg<true, 2, 2, 8, 8, 1, 32, 3, 2>;
+using SimtLargeDown = SimtCfg<false, 1, 2, 8, 8, 2, 32, 3, 2>;
+using SimtMidUp = SimtCfg<true, 1, 1, 8, 8, 4, 64, 2, 3>;
+using SimtMidDown = SimtCfg<false, 1, 1, 8, 8, 4, 64, 2, 3>;
+using SimtSmallUp = SimtCfg<true, 1, 1, 4, 4, 8, 256, 2, 1>;
+using SimtSmallDown = SimtCfg<false, 1, 1, 4, 4, 8, 256, 2, 1>;
+static_assert(SimtLargeUp::BR == simt_rows_up(SimtShape::kLarge) &&
+                  SimtLargeDown::BR == simt_rows_down(SimtShape::kLarge) &&
+                  SimtMidUp::BR == simt_rows_up(SimtShape::kMid) &&
+                  SimtMidDown::BR == simt_rows_down(SimtShape::kMid) &&
+                  SimtSmallUp::BR == simt_rows_up(SimtShape::kSmall) &&
+                  SimtSmallDown::BR == simt_rows_down(SimtShape::kSmall),
+              "row tiles the permute is told");
 
-__device__ __forceinline__ TileInfo find_tile(const GroupMap& gm, int u) {
-  TileInfo ti;
-  ti.ok = false;
+// The row tile of block u, found by one warp in two round trips: the group is the number of tile
+// prefixes at or below u (32 groups per step; loads bypass L1, which may hold an earlier call's).
+struct TileInfo {
+  int g, slot0, nrows;
+};
+template <int BR>
+__device__ __forceinline__ TileInfo find_tile(const GroupMap& gm, int u, int lane) {
+  const unsigned full = 0xffffffffu;
+  TileInfo ti{0, 0, 0};
   if (gm.tile_offs) {
-    if (u >= gm.tile_offs[gm.n_groups]) return ti;
-    int lo = 0, hi = gm.n_groups - 1;  // last g with tile_offs[g] <= u
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (gm.tile_offs[mid] <= u) lo = mid;
-      else hi = mid - 1;
+    const int G = gm.n_groups;
+    int cnt = 0, first = 0, beg = 0, end = 0;
+    for (int b = 0; b < G; b += 32) {
+      const int e = b + lane;
+      const int te = e < G ? __ldcg(gm.tile_offs + e) : 0x7fffffff;
+      const int oe = e < G ? __ldcg(gm.row_offs + e) : 0;
+      const int on = e < G ? __ldcg(gm.row_offs + e + 1) : 0;
+      const unsigned m = __ballot_sync(full, te <= u);
+      if (m) {  // (prefixes ascend: the last group at or below u is the highest set lane)
+        const int l = 31 - __clz(m);
+        first = __shfl_sync(full, te, l);
+        beg = __shfl_sync(full, oe, l);
+        end = __shfl_sync(full, on, l);
+      }
+      cnt += __popc(m);
     }
-    ti.g = lo;
-    ti.row0 = (u - gm.tile_offs[lo]) * BR;
+    ti.g = cnt - 1;
+    ti.slot0 = beg + (u - first) * BR;
+    ti.nrows = min(BR, end - ti.slot0);  // <= 0 past the last group's tiles
   } else {
     const int tpg = (gm.uniform_rows + BR - 1) / BR;
     if (u >= tpg * gm.n_groups) return ti;
     ti.g = u / tpg;
-    ti.row0 = (u % tpg) * BR;
+    const int r0 = (u - ti.g * tpg) * BR;
+    ti.slot0 = ti.g * gm.uniform_rows + r0;
+    ti.nrows = min(BR, gm.uniform_rows - r0);
   }
-  const int beg = gm.row_offs ? gm.row_offs[ti.g] : ti.g * gm.uniform_rows;
-  const int end = gm.row_offs ? gm.row_offs[ti.g + 1] : (ti.g + 1) * gm.uniform_rows;
-  ti.slot0 = beg + ti.row0;
-  ti.nrows = min(BR, end - ti.slot0);
-  ti.ok = ti.nrows > 0;
   return ti;
 }
 
 __device__ __forceinline__ int in_row(const GroupMap& gm, int g, int s) {
-  if (gm.row_mode == kRowGather) return gm.row_tok[s];
+  if (gm.row_mode == kRowGather) return __ldcg(gm.row_tok + s);
   if (gm.row_mode == kRowSlot) return s;
   return s - g * gm.uniform_rows;
 }
 
-template <typename TW, bool GATEUP>
-__global__ void __launch_bounds__(kThreads)
-ffn_simt_kernel(const TW* __restrict__ in, const TW* __restrict__ w0, const TW* __restrict__ w1,
-                int Fout, int Kdim, GroupMap gm, void* __restrict__ outp) {
-  __shared__ float as[BR][BK + 1];
-  __shared__ float ws0[BF][BK + 1];
-  __shared__ float ws1[GATEUP ? BF : 1][BK + 1];
-  __shared__ int rows[BR];
-  pdl_wait();
-  pdl_launch_dependents();
-  const TileInfo ti = find_tile(gm, blockIdx.y);
-  if (!ti.ok) return;
-  const int f0 = blockIdx.x * BF;
-  const int tid = threadIdx.x;
-  if (tid < BR) rows[tid] = tid < ti.nrows ? in_row(gm, ti.g, ti.slot0 + tid) : -1;
+template <class C>
+__global__ void __launch_bounds__(C::THREADS, C::MINB)
+ffn_simt_kernel(const float* __restrict__ in, const float* __restrict__ w0,
+                const float* __restrict__ w1, int Fout, int Kdim, GroupMap gm,
+                float* __restrict__ out) {
+  constexpr int BR = C::BR, BC = C::BC, BK = C::BK, LD = C::LD, ST = C::ST, TM = C::TM,
+                TN = C::TN, KG = C::KG, NT = C::THREADS;
+  constexpr int PIECES = BK / 4;          // 16-byte pieces of a chunk row
+  constexpr int HALF = 4 * TN;            // gate (then up) columns of a warp tile
+  extern __shared__ __align__(16) float smem_f[];
+  __shared__ TileInfo s_tile;
+  __shared__ int s_row[BR];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the gate/up launch follows the permute; the down launch is two launches behind it, so its
+  // tile and weights need not wait for the gate/up kernel
+  if (C::GATEUP) pdl_wait();
+  if (warp == 0) {
+    const TileInfo ti = find_tile<BR>(gm, blockIdx.y, lane);
+    if (lane == 0) s_tile = ti;
+    if (C::GATEUP || gm.row_mode != kRowGather)
+      for (int r = lane; r < BR; r += 32)
+        s_row[r] = ti.nrows > 0 ? in_row(gm, ti.g, ti.slot0 + min(r, ti.nrows - 1)) : 0;
+  }
   __syncthreads();
-  const size_t wbase = (size_t)ti.g * Fout * Kdim;
-  const int tr = tid >> 4;   // 0..15 -> rows tr, tr + 16
-  const int tf = tid & 15;   // 0..15 -> features tf + 16 q
-  float acc0[2][4] = {}, acc1[2][4] = {};
-  for (int k0 = 0; k0 < Kdim; k0 += BK) {
-    for (int i = tid; i < BR * BK; i += kThreads) {
-      const int r = i / BK, kk = i % BK;
-      const int row = rows[r];
-      as[r][kk] = row >= 0 ? ld(in, (size_t)row * Kdim + k0 + kk) : 0.f;
+  const TileInfo ti = s_tile;
+  if (ti.nrows <= 0) {
+    if (!C::GATEUP) pdl_wait();
+    pdl_launch_dependents();
+    return;
+  }
+  const int f0 = blockIdx.x * C::FEAT;
+  // weight row r of the block's tile: per warp column, HALF gate rows then HALF up rows of the
+  // same features, or consecutive down rows; rows past Fout repeat the last one (never stored)
+  auto w_row = [&](int r) -> const float* {
+    if (C::GATEUP) {
+      const int wc = r / (2 * HALF), q = r % (2 * HALF);
+      const int f = min(f0 + wc * HALF + q % HALF, Fout - 1);
+      return (q < HALF ? w0 : w1) + ((size_t)ti.g * Fout + f) * Kdim;
     }
-    for (int i = tid; i < BF * BK; i += kThreads) {
-      const int f = i / BK, kk = i % BK;
-      const bool okf = f0 + f < Fout;
-      ws0[f][kk] = okf ? ld(w0, wbase + (size_t)(f0 + f) * Kdim + k0 + kk) : 0.f;
-      if (GATEUP) ws1[f][kk] = okf ? ld(w1, wbase + (size_t)(f0 + f) * Kdim + k0 + kk) : 0.f;
+    return w0 + ((size_t)ti.g * Fout + min(f0 + r, Fout - 1)) * Kdim;
+  };
+  const int chunks = (Kdim + BK - 1) / BK;
+  // rows past the tile's repeat its last one (their outputs are never stored); K is a multiple of
+  // 64, and a last chunk shorter than BK is copied and summed up to K
+  auto load_w = [&](int c) {
+    float* st = smem_f + (c % ST) * C::STAGE + BR * LD;
+    const int k0 = c * BK, np = min(PIECES, (Kdim - k0) / 4);
+    for (int i = tid; i < BC * PIECES; i += NT) {
+      const int r = i / PIECES, p = i % PIECES;
+      if (p < np)
+        cp_async16((uint32_t)__cvta_generic_to_shared(st + r * LD + p * 4), w_row(r) + k0 + p * 4);
     }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < BK; ++kk) {
-      const float a0 = as[tr][kk], a1 = as[tr + 16][kk];
+  };
+  auto load_x = [&](int c) {
+    float* st = smem_f + (c % ST) * C::STAGE;
+    const int k0 = c * BK, np = min(PIECES, (Kdim - k0) / 4);
+    for (int i = tid; i < BR * PIECES; i += NT) {
+      const int r = i / PIECES, p = i % PIECES;
+      if (p < np)
+        cp_async16((uint32_t)__cvta_generic_to_shared(st + r * LD + p * 4),
+                   in + (size_t)s_row[r] * Kdim + k0 + p * 4);
+    }
+  };
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float b0 = ws0[tf + 16 * q][kk];
-        acc0[0][q] = fmaf(a0, b0, acc0[0][q]);
-        acc0[1][q] = fmaf(a1, b0, acc0[1][q]);
-        if (GATEUP) {
-          const float b1 = ws1[tf + 16 * q][kk];
-          acc1[0][q] = fmaf(a0, b1, acc1[0][q]);
-          acc1[1][q] = fmaf(a1, b1, acc1[1][q]);
+  for (int c = 0; c < ST - 1; ++c)
+    if (c < chunks) load_w(c);
+  if (!C::GATEUP) pdl_wait();
+  pdl_launch_dependents();
+#pragma unroll
+  for (int c = 0; c < ST - 1; ++c) {
+    if (c < chunks) load_x(c);
+    cp_async_commit();
+  }
+
+  const int kg = warp / (C::WR * C::WC), wt = warp % (C::WR * C::WC);
+  const int wr = wt / C::WC, wc = wt % C::WC;
+  const int lr = lane >> 3, lc = lane & 7;
+  float acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+  for (int c = 0; c < chunks; ++c) {
+    cp_async_wait<ST - 2>();
+    __syncthreads();  // chunk c is there for everyone, and chunk c - 1's buffer is free
+    if (c + ST - 1 < chunks) {
+      load_w(c + ST - 1);
+      load_x(c + ST - 1);
+    }
+    cp_async_commit();
+    const int kc = min(BK, Kdim - c * BK) / KG;  // this warp group's columns (K % 64 == 0)
+    const float* as = smem_f + (c % ST) * C::STAGE + (wr * 4 * TM + lr) * LD + kg * kc;
+    const float* bs = smem_f + (c % ST) * C::STAGE + (BR + wc * 8 * TN + lc) * LD + kg * kc;
+#pragma unroll 2
+    for (int kk = 0; kk < kc; kk += 4) {
+      float4 b[TN];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) b[j] = *(const float4*)(bs + 8 * j * LD + kk);
+#pragma unroll
+      for (int i = 0; i < TM; ++i) {
+        const float4 a = *(const float4*)(as + 4 * i * LD + kk);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          acc[i][j] = fmaf(a.x, b[j].x, acc[i][j]);
+          acc[i][j] = fmaf(a.y, b[j].y, acc[i][j]);
+          acc[i][j] = fmaf(a.z, b[j].z, acc[i][j]);
+          acc[i][j] = fmaf(a.w, b[j].w, acc[i][j]);
         }
       }
     }
-    __syncthreads();
   }
+  cp_async_wait<0>();
+
+  if constexpr (KG == 1) {
 #pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    const int r = tr + 16 * rr;
-    if (r >= ti.nrows) continue;
-    const size_t slot = (size_t)ti.slot0 + r;
+    for (int i = 0; i < TM; ++i) {
+      const int r = wr * 4 * TM + lr + 4 * i;
+      if (r >= ti.nrows) continue;
+      float* o = out + (size_t)(ti.slot0 + r) * Fout;
+      if constexpr (C::GATEUP) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int f = f0 + tf + 16 * q;
-      if (f >= Fout) continue;
-      if (GATEUP) {
-        const float g = acc0[rr][q];
-        const float silu = g / (1.0f + expf(-g));
-        st((TW*)outp, slot * Fout + f, silu * acc1[rr][q]);
+        for (int j = 0; j < TN / 2; ++j) {
+          const int f = f0 + wc * HALF + lc + 8 * j;
+          const float g = acc[i][j];
+          if (f < Fout) o[f] = g / (1.0f + expf(-g)) * acc[i][j + TN / 2];
+        }
       } else {
-        ((float*)outp)[slot * Fout + f] = acc0[rr][q];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          const int f = f0 + wc * 8 * TN + lc + 8 * j;
+          if (f < Fout) o[f] = acc[i][j];
+        }
       }
     }
+  } else {
+    // the warp groups' tiles into shared memory (the ring is no longer read), then their sums
+    constexpr int RL = BC + 1;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j)
+        smem_f[(kg * BR + wr * 4 * TM + lr + 4 * i) * RL + wc * 8 * TN + lc + 8 * j] = acc[i][j];
+    __syncthreads();
+    for (int q = tid; q < BR * C::FEAT; q += NT) {
+      const int r = q / C::FEAT, fl = q % C::FEAT, f = f0 + fl;
+      if (r >= ti.nrows || f >= Fout) continue;
+      // column of the feature's first (gate or only) weight row in the tile
+      const int col = C::GATEUP ? fl / HALF * (2 * HALF) + fl % HALF : fl;
+      float g = 0.f, u = 0.f;
+#pragma unroll
+      for (int s = 0; s < KG; ++s) {
+        g += smem_f[(s * BR + r) * RL + col];
+        if (C::GATEUP) u += smem_f[(s * BR + r) * RL + col + HALF];
+      }
+      out[(size_t)(ti.slot0 + r) * Fout + f] = C::GATEUP ? g / (1.0f + expf(-g)) * u : g;
+    }
   }
+}
+
+template <class C>
+cudaError_t launch_simt(const float* in, const float* w0, const float* w1, int Fout, int Kdim,
+                        const GroupMap& gm, float* out, cudaStream_t st) {
+  static std::once_flag once;
+  static cudaError_t attr_err = cudaSuccess;
+  std::call_once(once, [] {
+    attr_err = cudaFuncSetAttribute(ffn_simt_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    C::SMEM);
+  });
+  if (attr_err != cudaSuccess) return attr_err;
+  const dim3 grid((Fout + C::FEAT - 1) / C::FEAT, gm.max_tiles);
+  if (grid.y == 0) return cudaSuccess;
+  return launch_pdl(ffn_simt_kernel<C>, grid, dim3(C::THREADS), C::SMEM, st, in, w0, w1, Fout,
+                    Kdim, gm, out);
 }
 
 }  // namespace
 
-cudaError_t launch_ffn_gateup_simt(int dtype_bf16, const void* in, const void* wg, const void* wu,
-                                   int Fout, int Kdim, GroupMap gm, void* act, cudaStream_t st) {
-  dim3 grid((Fout + BF - 1) / BF, gm.max_tiles);
-  if (grid.y == 0) return cudaSuccess;
-  if (dtype_bf16)
-    return launch_pdl(ffn_simt_kernel<__nv_bfloat16, true>, grid, dim3(kThreads), 0, st,
-                      (const __nv_bfloat16*)in, (const __nv_bfloat16*)wg,
-                      (const __nv_bfloat16*)wu, Fout, Kdim, gm, act);
-  return launch_pdl(ffn_simt_kernel<float, true>, grid, dim3(kThreads), 0, st, (const float*)in,
-                    (const float*)wg, (const float*)wu, Fout, Kdim, gm, act);
+SimtShape simt_shape(int T, int K, int F) {
+  // selected rows x width: the lines of the table at the top of this file (512 and 1999 tokens)
+  const long long work = (long long)T * K * F;
+  return work >= 2000000 ? SimtShape::kLarge
+                         : work >= 512 * 1024 ? SimtShape::kMid : SimtShape::kSmall;
 }
 
-cudaError_t launch_ffn_down_simt(int dtype_bf16, const void* act, const void* wd, int Dout,
-                                 int Kdim, GroupMap gm, float* out, cudaStream_t st) {
-  dim3 grid((Dout + BF - 1) / BF, gm.max_tiles);
-  if (grid.y == 0) return cudaSuccess;
-  GroupMap g2 = gm;
-  g2.row_mode = kRowSlot;  // the down projection reads act rows in slot order
-  if (dtype_bf16)
-    return launch_pdl(ffn_simt_kernel<__nv_bfloat16, false>, grid, dim3(kThreads), 0, st,
-                      (const __nv_bfloat16*)act, (const __nv_bfloat16*)wd,
-                      (const __nv_bfloat16*)nullptr, Dout, Kdim, g2, (void*)out);
-  return launch_pdl(ffn_simt_kernel<float, false>, grid, dim3(kThreads), 0, st,
-                    (const float*)act, (const float*)wd, (const float*)nullptr, Dout, Kdim, g2,
-                    (void*)out);
+cudaError_t launch_ffn_gateup_simt(const float* in, const float* wg, const float* wu, int Fout,
+                                   int Kdim, GroupMap gm, SimtShape shape, float* act,
+                                   cudaStream_t st) {
+  if (shape == SimtShape::kLarge)
+    return launch_simt<SimtLargeUp>(in, wg, wu, Fout, Kdim, gm, act, st);
+  if (shape == SimtShape::kMid)
+    return launch_simt<SimtMidUp>(in, wg, wu, Fout, Kdim, gm, act, st);
+  return launch_simt<SimtSmallUp>(in, wg, wu, Fout, Kdim, gm, act, st);
+}
+
+cudaError_t launch_ffn_down_simt(const float* act, const float* wd, int Dout, int Kdim,
+                                 GroupMap gm, SimtShape shape, float* out, cudaStream_t st) {
+  gm.row_mode = kRowSlot;  // act rows are in slot order, the shared experts' too
+  if (shape == SimtShape::kLarge)
+    return launch_simt<SimtLargeDown>(act, wd, nullptr, Dout, Kdim, gm, out, st);
+  if (shape == SimtShape::kMid)
+    return launch_simt<SimtMidDown>(act, wd, nullptr, Dout, Kdim, gm, out, st);
+  return launch_simt<SimtSmallDown>(act, wd, nullptr, Dout, Kdim, gm, out, st);
 }
 
 }  // namespace eat

@@ -221,6 +221,19 @@ def test_k_equals_e():
     run_parity(sh, lw, [50, 50, 50])
 
 
+@pytest.mark.parametrize("d,F,E,K,S,Ts", [
+    (64, 64, 3, 1, 0, [1, 17, 2048]),       # one 64-column K chunk; one feature tile
+    (192, 320, 5, 2, 0, [100, 900, 3200]),  # small, mid and large shape; ragged last K chunk
+    (320, 192, 40, 3, 2, [15, 16, 1000, 3600]),  # more than 32 experts; shared experts
+])
+def test_fp32_shapes(d, F, E, K, S, Ts):
+    """fp32 layers through each of the three kernel shapes, at row tiles that are partial, full
+    and one past full, and widths that are not multiples of a block's feature tile."""
+    sh = W.scaled(W.TOY, f"f32-{d}", d_model=d, n_experts=E, d_ff=F, max_k=K, n_shared=S,
+                  d_ff_shared=F if S else 0)
+    run_parity(sh, W.make_layer(sh), Ts)
+
+
 @pytest.mark.parametrize("E,K,T", [(256, 8, 300), (100, 16, 130), (33, 5, 77)])
 def test_expert_counts_and_max_k(E, K, T):
     """Up to 256 experts (8 per lane of the selection warp), a ragged lane layout, K = 16."""
