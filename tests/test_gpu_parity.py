@@ -242,6 +242,33 @@ def test_expert_counts_and_max_k(E, K, T):
     run_parity(sh, lw, [T, 1, T // 3])
 
 
+@pytest.mark.parametrize("mode", ["eat", "topk"])
+@pytest.mark.parametrize("E,K", [(5, 3), (32, 16), (60, 8), (128, 5), (200, 16)])
+def test_k_cap_ties_go_to_lower_index(E, K, mode):
+    """Experts with identical router weights tie exactly: the K cap keeps the lower indices.  Three
+    distinct rows of W_r, so that ties straddle the cap whatever the order of the three."""
+    sh = W.scaled(W.OLMOE, f"ties{E}", d_model=128, n_experts=E, d_ff=64, max_k=K)
+    lw = W.make_layer(sh)
+    lw.w_router = lw.w_router[torch.arange(E) % 3].contiguous()
+    lw.b_router = torch.zeros_like(lw.b_router)
+    kw = {"alpha1": 0.0, "alpha2": 1e9, "clamp_enabled": 0}  # tau = 0: every expert is a candidate
+    if mode == "topk":
+        kw = {"router_mode": eat.EAT_ROUTER_TOPK}
+    L = eat.EatLayer.from_workload(lw, 300, gpu_params(sh, **kw))
+    for T in (7, 300):
+        x = W.make_tokens(sh, T, step=T).cuda()
+        idx, w, k = L.route(x, 0)
+        torch.cuda.synchronize()
+        p = orc.route(np64(x), oracle_layer(lw), orc.Accounts.zeros(E),
+                      oracle_params(sh, **kw), 0).p
+        # (the three logits are distinct to far more than fp32 rounding on these inputs)
+        g = np.round(p[:, :3] / 1e-9)
+        for t in range(T):
+            order = sorted(range(E), key=lambda e: (-g[t, e % 3], e))[:K]
+            assert idx[t, :k[t]].tolist() == sorted(order), t
+    L.close()
+
+
 @pytest.mark.parametrize("E,d", [(64, 256), (100, 192), (256, 512)])
 def test_router_runs_split_between_blocks(E, d):
     """Router scores of calls above 128 tokens: a persistent grid takes equal runs of
