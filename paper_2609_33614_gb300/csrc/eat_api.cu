@@ -211,6 +211,13 @@ eat_status run_route(eat_handle* h, const void* x, int T, int ppl_sign, int32_t*
     rp.tau_in = h->tau_state;
     rp.tau_out = write_tau ? h->tau_state : nullptr;
   }
+  const void* xr = x_host ? x_host : x;
+  if (route_fused(xr, h->bf16, h->desc.w_router, T, h->d, h->E))
+    return launch(h, kRoute, st, "route", [&] {
+      return launch_route_fused(xr, h->bf16, h->desc.w_router, h->desc.b_router, T, h->d, h->E,
+                                h->K, h->N, h->P, h->C, rp, idx, w, k, psel, st,
+                                x_host ? const_cast<void*>(x) : nullptr);
+    });
   const int split = router_split(T, h->d, h->E);
   EAT_TRY(launch(h, kRoute, st, "router logits", [&] {
     if (x_host)
@@ -675,7 +682,7 @@ static eat_status forward_host(eat_handle* h, const void* x_host, int32_t T, int
   void* xd = h->backend == 1 ? mapped_host(x_host) : nullptr;
   void* yd = xd ? mapped_host(y_host) : nullptr;
   if (xd && yd && ((uintptr_t)xd & 15) == 0 && ((uintptr_t)yd & 15) == 0 &&
-      router_copies_x(xd, h->bf16, h->desc.w_router, T, h->d) &&
+      router_copies_x(xd, h->bf16, h->desc.w_router, T, h->d, h->E) &&
       !shared_on_side_stream(h, T, tc_tile_rows(h->tc, T))) {
     // a call on another stream may still read this staging buffer
     e = cudaStreamWaitEvent(st, h->ev_done[i], 0);

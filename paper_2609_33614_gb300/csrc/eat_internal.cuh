@@ -72,6 +72,27 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, ((KArgs)args)...);
 }
 
+// The same with clusters of `cluster` CTAs along x.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, int cluster, dim3 block,
+                               size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = pdl_enabled() ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, ((KArgs)args)...);
+}
+
 constexpr int kMaxExperts = 256;
 constexpr int kMaxK = 16;
 
@@ -99,7 +120,15 @@ struct RouteParams {
 cudaError_t launch_router_logits(const void* x, int x_bf16, const float* w_router, int T, int d,
                                  int E, int n_split, float2* part, cudaStream_t st,
                                  void* xcopy = nullptr);
-bool router_copies_x(const void* x, int x_bf16, const float* w_router, int T, int d);
+bool router_copies_x(const void* x, int x_bf16, const float* w_router, int T, int d, int E);
+// Scores and selection in one launch, without scratch, for the calls for which route_fused holds
+// (x, w_router: their alignment); xcopy as above.
+bool route_fused(const void* x, int x_bf16, const float* w_router, int T, int d, int E);
+cudaError_t launch_route_fused(const void* x, int x_bf16, const float* w_router,
+                               const float* b_router, int T, int d, int E, int K,
+                               const int64_t* accN, const double* accP, const double* accC,
+                               RouteParams rp, int32_t* idx, float* w, int32_t* k, float* psel,
+                               cudaStream_t st, void* xcopy = nullptr);
 // Warp-per-token softmax + history score + threshold + selection + renormalisation; the router
 // scores are the sum over the n_split slices of part ([split][T][E] fp32 pairs).
 cudaError_t launch_route_select(const float2* part, int n_split, const float* b_router, int T,

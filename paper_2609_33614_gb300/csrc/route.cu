@@ -1,6 +1,8 @@
 // Router and EAT selection (§3.1-§3.4 of the EAT paper, Eq. 1-8).
 //
-//  router_logits_small_kernel (T <= 128, decode) / router_logits_sk_kernel (bf16 x, larger calls;
+//  route_fused_kernel (T <= 128 and d <= 4096, and some larger calls): scores and selection of a
+//      small call in one launch, a cluster of CTAs per group of tokens.
+//  router_logits_small_kernel (T <= 128, d > 4096) / router_logits_sk_kernel (bf16 x, larger calls;
 //      stream-K over tiles and chunks of d) / router_logits_kernel (other large calls; both tiled
 //      through shared memory): partial router scores x . w_r over slices of d: fp32 FMA inside
 //      16- or 32-wide chunks, chunk sums accumulated in Kahan-compensated fp32, so the
@@ -202,7 +204,11 @@ router_logits_small_kernel(const TX* __restrict__ x, const float* __restrict__ w
 // two units ahead; one block barrier per unit.
 constexpr int kSKT = 64, kSKE = 64, kSKS = kChunkK + 4, kSKStages = 3;
 constexpr int kSKTM = 4;        // tokens per thread: 256 threads, two CTAs per SM
-constexpr int kSKMinUnits = 8;  // 256 columns of d per CTA at least
+// Columns of d per CTA at least: 256, or 128 while the grid is no larger than the SM count (more CTAs
+// cut the run of a call that does not fill the GPU; beyond that the selection loses more to the
+// slices).  OLMoE router, us per routing call with 256 / 128: 200 tokens 18.5 / 14.4, 512 18.5 /
+// 15.6, 1000 19.4 / 23.1 (there with twice the SMs).
+constexpr int kSKMinUnits = 8, kSKMinUnitsSmall = 4;
 constexpr size_t kSKSmem = (size_t)kSKStages * (kSKT + kSKE) * kSKS * sizeof(float);
 template <int TM>
 struct SkCfg {
@@ -399,63 +405,62 @@ __device__ __forceinline__ float warp_max(float v) {
 
 constexpr int kSelectThreads = 256;
 
-// S_h (Eq. 1) for all experts into smem, readings: empty-history terms are 0; c_mode 0 uses
-// C_i / sum C, c_mode 1 the raw C_i.  sum N is exact (int64), sum C a compensated fp32 sum of the
-// fp32-rounded C_i; the three ratios are fp32 divisions (relative error ~3e-7, far inside the
+// S_h (Eq. 1) for all experts into smem, by one warp, readings: empty-history terms are 0; c_mode 0
+// uses C_i / sum C, c_mode 1 the raw C_i.  sum N is exact (int64), sum C a compensated fp32 sum of
+// the fp32-rounded C_i; the three ratios are fp32 divisions (relative error ~3e-7, far inside the
 // 1e-5 margin at which a token's selection counts as decided).  No fp64 arithmetic: it would run
 // on GB300's narrow fp64 pipe in every block.  The selection kernel runs this before its
 // dependency wait: the accounts are at least two launches old (the router-score kernel comes
-// between), and every kernel lets its dependent start only after its own wait.  The loads bypass
-// L1 (ld.global.cg), which may still hold an earlier call's lines before the wait.
-__device__ void history_score_block(const int64_t* accN, const double* accP, const double* accC,
-                                    int E, const RouteParams& rp, float* s_h) {
-  __shared__ long long red_n[kSelectThreads / 32];
-  __shared__ float red_c[2][kSelectThreads / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  long long n_sum = 0;
-  float c_hi = 0.f, c_lo = 0.f;
-  for (int e = tid; e < E; e += blockDim.x) {
-    n_sum += (long long)__ldcg(accN + e);
-    df_add(c_hi, c_lo, (float)__ldcg(accC + e));
+// between), and every kernel lets its dependent start only after its own wait; the one-launch
+// kernel of small calls runs it after its wait.  The loads bypass L1 (ld.global.cg), which may
+// still hold an earlier call's lines before the wait.
+template <int EPL>
+__device__ __forceinline__ void history_scores(const int64_t* accN, const double* accP,
+                                               const double* accC, int E, const RouteParams& rp,
+                                               float* s_h, int lane) {
+  const unsigned full = 0xffffffffu;
+  long long n[EPL], n_sum = 0;
+  float pe[EPL], ce[EPL], h[EPL], l[EPL];
+#pragma unroll
+  for (int i = 0; i < EPL; ++i) {
+    const int e = lane + 32 * i;
+    n[i] = e < E ? (long long)__ldcg(accN + e) : 0;
+    pe[i] = e < E ? (float)__ldcg(accP + e) : 0.f;
+    ce[i] = e < E ? (float)__ldcg(accC + e) : 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < EPL; ++i) {
+    n_sum += n[i];
+    h[i] = 0.f;
+    l[i] = 0.f;
+    df_add(h[i], l[i], ce[i]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    n_sum += __shfl_xor_sync(0xffffffffu, n_sum, o);
-    const float oh = __shfl_xor_sync(0xffffffffu, c_hi, o);
-    const float ol = __shfl_xor_sync(0xffffffffu, c_lo, o);
-    df_add(c_hi, c_lo, oh, ol);
-  }
-  if (lane == 0) {
-    red_n[warp] = n_sum;
-    red_c[0][warp] = c_hi;
-    red_c[1][warp] = c_lo;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    long long a = 0;
-    float bh = 0.f, bl = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      a += red_n[w];
-      df_add(bh, bl, red_c[0][w], red_c[1][w]);
+    n_sum += __shfl_xor_sync(full, n_sum, o);
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) {
+      const float oh = __shfl_xor_sync(full, h[i], o);
+      const float ol = __shfl_xor_sync(full, l[i], o);
+      df_add(h[i], l[i], oh, ol);
     }
-    red_n[0] = a;
-    red_c[0][0] = bh + bl;
   }
-  __syncthreads();
-  const float total_n = (float)red_n[0];
-  const float total_c = red_c[0][0];
-  for (int e = tid; e < E; e += blockDim.x) {
-    const long long ni = __ldcg(accN + e);
-    const float n = (float)ni;
-    const float a = ni > 0 ? n / total_n : 0.f;
-    const float b = ni > 0 ? (float)__ldcg(accP + e) / n : 0.f;
-    const float ce = (float)__ldcg(accC + e);
+  float c_hi = 0.f, c_lo = 0.f;
+#pragma unroll
+  for (int i = 0; i < EPL; ++i)
+    df_add(c_hi, c_lo, __shfl_sync(full, h[i], 0), __shfl_sync(full, l[i], 0));
+  const float total_n = (float)n_sum, total_c = c_hi + c_lo;
+#pragma unroll
+  for (int i = 0; i < EPL; ++i) {
+    const int e = lane + 32 * i;
+    const float nf = (float)n[i];
+    const float a = n[i] > 0 ? nf / total_n : 0.f;
+    const float b = n[i] > 0 ? pe[i] / nf : 0.f;
     float c;
-    if (rp.c_mode == EAT_C_RAW) c = ce;
-    else c = total_c > 0.f ? ce / total_c : 0.f;
-    s_h[e] = rp.w1 * a + rp.w2 * b + rp.w3 * c;
+    if (rp.c_mode == EAT_C_RAW) c = ce[i];
+    else c = total_c > 0.f ? ce[i] / total_c : 0.f;
+    if (e < E) s_h[e] = rp.w1 * a + rp.w2 * b + rp.w3 * c;
   }
-  __syncthreads();
 }
 
 // Warp-wide bitonic sort of the 32 x EPL values a warp holds (element j * 32 + lane in register j
@@ -522,61 +527,41 @@ __device__ __forceinline__ void keep_first(const float (&v)[EPL], const bool (&i
   }
 }
 
+// The selection's inputs and outputs besides the scores.
+struct SelectArgs {
+  const float* bias;   // [E] or null
+  int T, E, K;
+  const int64_t* accN;
+  const double *accP, *accC;
+  RouteParams rp;
+  float inv_temp;
+  int32_t* out_idx;
+  float* out_w;
+  int32_t* out_k;
+  float* out_p;
+};
+
+// One warp: the selection of token t from its router scores x . w_r (compensated pairs hi, lo of
+// experts lane + 32 i) and biases bv; s_h: the history scores of all experts (shared memory).
 template <int EPL>
-__global__ void __launch_bounds__(kSelectThreads)
-route_select_kernel(const float2* __restrict__ part, int n_split, const float* __restrict__ bias,
-                    int T, int E, int K, const int64_t* __restrict__ accN,
-                    const double* __restrict__ accP, const double* __restrict__ accC,
-                    RouteParams rp, float inv_temp, int32_t* __restrict__ out_idx,
-                    float* __restrict__ out_w, int32_t* __restrict__ out_k,
-                    float* __restrict__ out_p) {
-  __shared__ float s_h[kMaxExperts];
-  history_score_block(accN, accP, accC, E, rp, s_h);
-  pdl_wait();
-  pdl_launch_dependents();
-
-  const int lane = threadIdx.x & 31;
-  const int warps = blockDim.x >> 5;
-  const int t = blockIdx.x * warps + (threadIdx.x >> 5);
-  if (t >= T) return;
+__device__ __forceinline__ void select_token(int t, float (&hi)[EPL], float (&lo)[EPL],
+                                             const float (&bv)[EPL], const float* s_h,
+                                             const SelectArgs& a, int lane) {
   const unsigned full = 0xffffffffu;
+  const int E = a.E, K = a.K;
+  const RouteParams& rp = a.rp;
   const float inv_e = 1.0f / (float)E;
-
   float p[EPL], I[EPL];
   bool valid[EPL];
-  float hi[EPL], lo[EPL], bv[EPL];
 #pragma unroll
-  for (int i = 0; i < EPL; ++i) {
-    const int e = lane + 32 * i;
-    valid[i] = e < E;
-    hi[i] = 0.f;
-    lo[i] = 0.f;
-    bv[i] = bias && valid[i] ? bias[e] : 0.f;
-  }
-  // the score partials in slice order, a chunk of slices' loads in flight before their sums
-  constexpr int kChunk = EPL <= 2 ? 8 : (EPL <= 4 ? 4 : 2);
-  for (int sp0 = 0; sp0 < n_split; sp0 += kChunk) {
-    float2 v[kChunk][EPL];
-#pragma unroll
-    for (int c = 0; c < kChunk; ++c)
-#pragma unroll
-      for (int i = 0; i < EPL; ++i)
-        v[c][i] = sp0 + c < n_split && valid[i]
-                      ? part[((size_t)(sp0 + c) * T + t) * E + lane + 32 * i]
-                      : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int c = 0; c < kChunk; ++c)
-#pragma unroll
-      for (int i = 0; i < EPL; ++i)
-        if (sp0 + c < n_split && valid[i]) df_add(hi[i], lo[i], v[c][i].x, v[c][i].y);
-  }
+  for (int i = 0; i < EPL; ++i) valid[i] = lane + 32 * i < E;
   float lmax = -INFINITY;
 #pragma unroll
   for (int i = 0; i < EPL; ++i) {
     float z = -INFINITY;
     if (valid[i]) {
-      if (bias) df_add(hi[i], lo[i], bv[i]);
-      z = (hi[i] + lo[i]) * inv_temp;
+      if (a.bias) df_add(hi[i], lo[i], bv[i]);
+      z = (hi[i] + lo[i]) * a.inv_temp;
     }
     p[i] = z;
     lmax = fmaxf(lmax, z);
@@ -757,18 +742,224 @@ route_select_kernel(const float2* __restrict__ part, int n_split, const float* _
     const unsigned b = __ballot_sync(full, sel[i]);
     if (sel[i]) {
       const int pos = base + __popc(b & lt);
-      out_idx[row + pos] = lane + 32 * i;
-      out_w[row + pos] = p[i] / denom;
-      if (out_p) out_p[row + pos] = p[i];
+      a.out_idx[row + pos] = lane + 32 * i;
+      a.out_w[row + pos] = p[i] / denom;
+      if (a.out_p) a.out_p[row + pos] = p[i];
     }
     base += __popc(b);
   }
   if (lane >= base && lane < K) {
-    out_idx[row + lane] = -1;
-    out_w[row + lane] = 0.f;
-    if (out_p) out_p[row + lane] = 0.f;
+    a.out_idx[row + lane] = -1;
+    a.out_w[row + lane] = 0.f;
+    if (a.out_p) a.out_p[row + lane] = 0.f;
   }
-  if (lane == 0) out_k[t] = base;
+  if (lane == 0) a.out_k[t] = base;
+}
+
+template <int EPL>
+__global__ void __launch_bounds__(kSelectThreads)
+route_select_kernel(const float2* __restrict__ part, int n_split, const SelectArgs a) {
+  __shared__ float s_h[kMaxExperts];
+  if (threadIdx.x < 32) history_scores<EPL>(a.accN, a.accP, a.accC, a.E, a.rp, s_h, threadIdx.x);
+  pdl_wait();
+  pdl_launch_dependents();
+  __syncthreads();
+
+  const int lane = threadIdx.x & 31;
+  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int T = a.T, E = a.E;
+  if (t >= T) return;
+  bool valid[EPL];
+  float hi[EPL], lo[EPL], bv[EPL];
+#pragma unroll
+  for (int i = 0; i < EPL; ++i) {
+    const int e = lane + 32 * i;
+    valid[i] = e < E;
+    hi[i] = 0.f;
+    lo[i] = 0.f;
+    bv[i] = a.bias && valid[i] ? a.bias[e] : 0.f;
+  }
+  // the score partials in slice order, a chunk of slices' loads in flight before their sums
+  constexpr int kChunk = EPL <= 2 ? 8 : (EPL <= 4 ? 4 : 2);
+  for (int sp0 = 0; sp0 < n_split; sp0 += kChunk) {
+    float2 v[kChunk][EPL];
+#pragma unroll
+    for (int c = 0; c < kChunk; ++c)
+#pragma unroll
+      for (int i = 0; i < EPL; ++i)
+        v[c][i] = sp0 + c < n_split && valid[i]
+                      ? part[((size_t)(sp0 + c) * T + t) * E + lane + 32 * i]
+                      : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int c = 0; c < kChunk; ++c)
+#pragma unroll
+      for (int i = 0; i < EPL; ++i)
+        if (sp0 + c < n_split && valid[i]) df_add(hi[i], lo[i], v[c][i].x, v[c][i].y);
+  }
+  select_token<EPL>(t, hi, lo, bv, s_h, a, lane);
+}
+
+// Small calls: scores and selection in one launch.  A cluster of one CTA per 512-column slice of d
+// takes TT tokens: each CTA computes its slice's scores of all experts into its shared memory (the
+// sums and order of router_logits_small_kernel; a warp takes Q = four (expert, token) pairs at a
+// time, so that the compensated sums over its lanes run side by side), and after a cluster barrier
+// a warp per token adds the slices in slice order (distributed shared memory) and selects.  One
+// more warp computes the history scores meanwhile.  What bounds it is latency: one launch, no L2
+// round trip of the scores, no scratch.  TT = 1 while that grid fits the SMs once; TT = 4 reads W_r
+// from L2 once for four tokens.  Up to 32 experts (EPL = 1), eight warps take one expert each and
+// registers are bounded so that three CTAs share an SM (a second wave of clusters of eight took
+// 9.1 us instead of 5.6 at 16 tokens).  us per routing call (graph of 10), two kernels / this one:
+// OLMoE 32 tokens 7.0 / 6.2, 128 12.3 / 8.1, 1 5.4 / 6.0; Mixtral 1 6.4 / 4.6, 64 7.5 / 6.0, 300
+// 20.3 / 13.5; the fp32 toy layer 64 5.8 / 4.7, 1999 19.9 / 12.0.
+constexpr int kFusedSlice = 512;
+constexpr int kFusedMaxSlices = 8;  // portable cluster size
+// Warps that compute scores: 16 take the 64 experts of one token in one round.
+template <int EPL>
+constexpr int kFusedWarps = EPL == 1 ? 8 : 16;
+template <int EPL>
+constexpr int kFusedThreads = 32 * (kFusedWarps<EPL> + 1);
+template <int EPL, int TT>
+constexpr int kFusedPairs = EPL == 1 && TT == 1 ? 1 : 4;  // Q
+
+__device__ __forceinline__ float2 ld_cluster_f2(const float2* p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(a)
+               : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
+               ::: "memory");
+}
+
+template <typename TX, int EPL, int TT>
+__global__ void __launch_bounds__(kFusedThreads<EPL>, EPL == 1 ? 3 : 1)
+route_fused_kernel(const TX* __restrict__ x, const float* __restrict__ wr, int d, const SelectArgs a,
+                   TX* __restrict__ xcopy) {
+  using X4 = decltype(load_x4((const TX*)nullptr));
+  constexpr int kVecs = kFusedSlice / 4;  // 4-element pieces of a slice row
+  constexpr int kWarps = kFusedWarps<EPL>, kThreads = kFusedThreads<EPL>;
+  constexpr int Q = kFusedPairs<EPL, TT>, EB = Q / TT;  // pairs and experts of a warp's round
+  extern __shared__ __align__(16) float2 s_part[];  // [TT][E]
+  __shared__ X4 xs[TT][kVecs];
+  __shared__ float s_h[kMaxExperts];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int s = blockIdx.x, nsl = gridDim.x, t0 = blockIdx.y * TT;  // cluster rank = slice
+  const int beg = s * kFusedSlice, len = min(kFusedSlice, d - beg);
+  const int E = a.E;
+  pdl_wait();
+  pdl_launch_dependents();
+  // the first round's weight rows are in flight while x is fetched
+  float4 w[EB][4];
+  auto load_w = [&](int e0) {
+#pragma unroll
+    for (int b = 0; b < EB; ++b)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int c = lane * 4 + 128 * i, e = e0 + b * kWarps;
+        w[b][i] = e < E && c < len ? *(const float4*)(wr + (size_t)e * d + beg + c)
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+  };
+  if (warp < kWarps) load_w(warp);
+  for (int q = tid; q < TT * kVecs; q += kThreads) {
+    const int j = q / kVecs, c = (q % kVecs) * 4;
+    X4 v;
+    memset(&v, 0, sizeof(v));
+    if (t0 + j < a.T && c < len) {
+      const size_t at = (size_t)(t0 + j) * d + beg + c;
+      v = load_x4(x + at);
+      if (xcopy) store_x4(xcopy + at, v);
+    }
+    xs[j][q % kVecs] = v;
+  }
+  __syncthreads();
+  if (warp == kWarps) {
+    history_scores<EPL>(a.accN, a.accP, a.accC, E, a.rp, s_h, lane);
+  } else {
+    for (int e0 = warp; e0 < E; e0 += EB * kWarps) {
+      if (e0 != warp) load_w(e0);
+      float hi[Q], lo[Q];  // pair b * TT + j: expert e0 + b kWarps, token j
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        const int b = q / TT, j = q % TT;
+        float acc = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 xv = xs[j][lane + 32 * i].val();
+          acc = fmaf(xv.x, w[b][i].x, acc);
+          acc = fmaf(xv.y, w[b][i].y, acc);
+          acc = fmaf(xv.z, w[b][i].z, acc);
+          acc = fmaf(xv.w, w[b][i].w, acc);
+        }
+        hi[q] = 0.f;
+        lo[q] = 0.f;
+        df_add(hi[q], lo[q], acc);
+      }
+      // compensated sum over the lanes (a fixed tree, the lower lane's pair first); a lane keeps
+      // half of the pairs it has left and sends its values of the others
+#pragma unroll
+      for (int m = 16, n = Q / 2; m > 0; m >>= 1, n >>= 1) {
+        const bool upper = (lane & m) != 0;
+        if (n > 0) {
+#pragma unroll
+          for (int q = 0; q < Q / 2; ++q) {
+            if (q < n) {
+              const float oh = __shfl_xor_sync(0xffffffffu, upper ? hi[q] : hi[q + n], m);
+              const float ol = __shfl_xor_sync(0xffffffffu, upper ? lo[q] : lo[q + n], m);
+              const float kh = upper ? hi[q + n] : hi[q], kl = upper ? lo[q + n] : lo[q];
+              hi[q] = upper ? oh : kh;
+              lo[q] = upper ? ol : kl;
+              df_add(hi[q], lo[q], upper ? kh : oh, upper ? kl : ol);
+            }
+          }
+        } else {
+          const float oh = __shfl_xor_sync(0xffffffffu, hi[0], m);
+          const float ol = __shfl_xor_sync(0xffffffffu, lo[0], m);
+          const float kh = hi[0], kl = lo[0];
+          hi[0] = upper ? oh : kh;
+          lo[0] = upper ? ol : kl;
+          df_add(hi[0], lo[0], upper ? kh : oh, upper ? kl : ol);
+        }
+      }
+      // (Q = 4: lane bits 4 and 3 picked pair lane / 8)
+      const int q = Q == 1 ? 0 : lane >> 3, e = e0 + q / TT * kWarps;
+      if ((lane & (Q == 1 ? 31 : 7)) == 0 && e < E) s_part[q % TT * E + e] = make_float2(hi[0], lo[0]);
+    }
+  }
+  cluster_barrier();
+  // token j's selection: warp j / nsl of the CTA of rank j % nsl
+  const int j = warp * nsl + s;
+  if (j < TT && t0 + j < a.T) {
+    float hi[EPL], lo[EPL], bv[EPL];
+#pragma unroll
+    for (int i = 0; i < EPL; ++i) {
+      const int e = lane + 32 * i;
+      hi[i] = 0.f;
+      lo[i] = 0.f;
+      bv[i] = a.bias && e < E ? a.bias[e] : 0.f;
+    }
+    constexpr int kChunk = EPL <= 2 ? 8 : (EPL <= 4 ? 4 : 2);  // slices in flight
+    for (int r0 = 0; r0 < nsl; r0 += kChunk) {
+      float2 v[kChunk][EPL];
+#pragma unroll
+      for (int c = 0; c < kChunk; ++c)
+#pragma unroll
+        for (int i = 0; i < EPL; ++i)
+          if (r0 + c < nsl && lane + 32 * i < E)
+            v[c][i] = ld_cluster_f2(&s_part[j * E + lane + 32 * i], r0 + c);
+#pragma unroll
+      for (int c = 0; c < kChunk; ++c)
+#pragma unroll
+        for (int i = 0; i < EPL; ++i)
+          if (r0 + c < nsl && lane + 32 * i < E) df_add(hi[i], lo[i], v[c][i].x, v[c][i].y);
+    }
+    select_token<EPL>(t0 + j, hi, lo, bv, s_h, a, lane);
+  }
+  cluster_barrier();  // no CTA leaves while another may read its scores
 }
 
 }  // namespace
@@ -818,6 +1009,7 @@ bool sk_plan(int T, int d, int E, int cap, SkPlan& out) {
   const long long tiles = (long long)((T + kSKT - 1) / kSKT) * ((E + kSKE - 1) / kSKE);
   const long long U = tiles * nc;
   long long G = std::min<long long>((long long)sms * per_sm, U / kSKMinUnits);
+  G = std::max(G, std::min<long long>(sms, U / kSKMinUnitsSmall));
   G = std::max<long long>(1, std::min(G, U));
   auto bound = [&](long long g) {
     const long long m = U / g;
@@ -855,15 +1047,28 @@ int router_split(int T, int d, int E) {
   return split;
 }
 
-bool router_copies_x(const void* x, int x_bf16, const float* w_router, int T, int d) {
-  const bool vec_ok = d % 4 == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)w_router & 15) == 0;
-  return vec_ok && (T <= kSmallT || (x_bf16 && sk_eligible(T, d)));
+static bool router_vec_ok(const void* x, const float* w_router, int d) {
+  return d % 4 == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)w_router & 15) == 0;
+}
+
+// One launch for scores and selection: every call of up to kSmallT tokens (d up to 4096, a cluster
+// of at most eight slices), and larger ones of fp32 x or few experts, where the tiled kernels'
+// 64-expert tiles would be mostly empty (Mixtral's 8 experts, us per routing call tiled / fused: 300
+// tokens 20.3 / 13.5, 500 20.7 / 19.7, 1000 28.6 / 42; OLMoE's 64: 200 tokens 14.4 / 16.8).
+bool route_fused(const void* x, int x_bf16, const float* w_router, int T, int d, int E) {
+  return router_vec_ok(x, w_router, d) && d <= kFusedSlice * kFusedMaxSlices &&
+         (T <= kSmallT || !x_bf16 || (long long)T * E <= 4096);
+}
+
+bool router_copies_x(const void* x, int x_bf16, const float* w_router, int T, int d, int E) {
+  return router_vec_ok(x, w_router, d) &&
+         (T <= kSmallT || (x_bf16 && sk_eligible(T, d)) || route_fused(x, x_bf16, w_router, T, d, E));
 }
 
 cudaError_t launch_router_logits(const void* x, int x_bf16, const float* w_router, int T, int d,
                                  int E, int n_split, float2* part, cudaStream_t st, void* xcopy) {
-  const bool vec_ok = d % 4 == 0 && ((uintptr_t)x & 15) == 0 && ((uintptr_t)w_router & 15) == 0;
-  if (xcopy && (!router_copies_x(x, x_bf16, w_router, T, d) || ((uintptr_t)xcopy & 15) != 0))
+  const bool vec_ok = router_vec_ok(x, w_router, d);
+  if (xcopy && (!router_copies_x(x, x_bf16, w_router, T, d, E) || ((uintptr_t)xcopy & 15) != 0))
     return cudaErrorInvalidValue;
   if (T <= kSmallT && vec_ok) {
     int per = (d + n_split - 1) / n_split;
@@ -894,21 +1099,63 @@ cudaError_t launch_router_logits(const void* x, int x_bf16, const float* w_route
                     (const float*)x, w_router, T, d, E, per, part);
 }
 
+static SelectArgs select_args(const float* b_router, int T, int E, int K, const int64_t* accN,
+                              const double* accP, const double* accC, const RouteParams& rp,
+                              int32_t* idx, float* w, int32_t* k, float* psel) {
+  return SelectArgs{b_router, T, E, K, accN, accP, accC, rp,
+                    (float)(1.0 / (double)rp.temperature), idx, w, k, psel};
+}
+
 cudaError_t launch_route_select(const float2* part, int n_split, const float* b_router, int T,
                                 int E, int K, const int64_t* accN, const double* accP,
                                 const double* accC, RouteParams rp, int32_t* idx, float* w,
                                 int32_t* k, float* psel, cudaStream_t st) {
   const int warps = kSelectThreads / 32;
   dim3 grid((T + warps - 1) / warps);
-  const float inv_temp = (float)(1.0 / (double)rp.temperature);
-#define EAT_SELECT(EPL)                                                                    \
-  launch_pdl(route_select_kernel<EPL>, grid, dim3(kSelectThreads), 0, st, part, n_split,    \
-             b_router, T, E, K, accN, accP, accC, rp, inv_temp, idx, w, k, psel)
+  const SelectArgs a = select_args(b_router, T, E, K, accN, accP, accC, rp, idx, w, k, psel);
+#define EAT_SELECT(EPL) \
+  launch_pdl(route_select_kernel<EPL>, grid, dim3(kSelectThreads), 0, st, part, n_split, a)
   if (E <= 32) return EAT_SELECT(1);
   if (E <= 64) return EAT_SELECT(2);
   if (E <= 128) return EAT_SELECT(4);
   return EAT_SELECT(8);
 #undef EAT_SELECT
+}
+
+namespace {
+template <typename TX, int EPL>
+cudaError_t launch_fused_t(const TX* x, const float* wr, int d, const SelectArgs& a, TX* xcopy,
+                           cudaStream_t st) {
+  int sms = 0, per_sm = 0;
+  if (!sk_device(sms, per_sm)) return cudaErrorInvalidDevice;
+  const int nsl = (d + kFusedSlice - 1) / kFusedSlice;
+  if (a.T * nsl <= sms)
+    return launch_pdl_cluster(route_fused_kernel<TX, EPL, 1>, dim3(nsl, a.T), nsl,
+                              dim3(kFusedThreads<EPL>), sizeof(float2) * a.E, st, x, wr, d, a, xcopy);
+  return launch_pdl_cluster(route_fused_kernel<TX, EPL, 4>, dim3(nsl, (a.T + 3) / 4), nsl,
+                            dim3(kFusedThreads<EPL>), sizeof(float2) * 4 * a.E, st, x, wr, d, a, xcopy);
+}
+template <typename TX>
+cudaError_t launch_fused_x(const TX* x, const float* wr, int d, const SelectArgs& a, TX* xcopy,
+                           cudaStream_t st) {
+  if (a.E <= 32) return launch_fused_t<TX, 1>(x, wr, d, a, xcopy, st);
+  if (a.E <= 64) return launch_fused_t<TX, 2>(x, wr, d, a, xcopy, st);
+  if (a.E <= 128) return launch_fused_t<TX, 4>(x, wr, d, a, xcopy, st);
+  return launch_fused_t<TX, 8>(x, wr, d, a, xcopy, st);
+}
+}  // namespace
+
+cudaError_t launch_route_fused(const void* x, int x_bf16, const float* w_router,
+                               const float* b_router, int T, int d, int E, int K,
+                               const int64_t* accN, const double* accP, const double* accC,
+                               RouteParams rp, int32_t* idx, float* w, int32_t* k, float* psel,
+                               cudaStream_t st, void* xcopy) {
+  if (!route_fused(x, x_bf16, w_router, T, d, E) || ((uintptr_t)xcopy & 15) != 0)
+    return cudaErrorInvalidValue;
+  const SelectArgs a = select_args(b_router, T, E, K, accN, accP, accC, rp, idx, w, k, psel);
+  if (x_bf16)
+    return launch_fused_x((const __nv_bfloat16*)x, w_router, d, a, (__nv_bfloat16*)xcopy, st);
+  return launch_fused_x((const float*)x, w_router, d, a, (float*)xcopy, st);
 }
 
 }  // namespace eat

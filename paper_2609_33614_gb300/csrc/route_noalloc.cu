@@ -130,13 +130,6 @@ extern "C" eat_status eat_route_noalloc(const void* x, int32_t T, int32_t d_mode
     return bad("eat_route_noalloc: T * n_experts exceeds the 131072 router scores its fixed "
                "1 MiB scratch holds; split the call into smaller token batches");
 
-  float2* scratch = nullptr;
-  const eat_status s = scratch_address(&scratch);
-  if (s != EAT_OK) return s;
-
-  int split = eat::router_split(T, d_model, n_experts);
-  while (split > 1 && (size_t)split * T * n_experts > kScratchScores) split /= 2;
-
   eat::RouteParams rp;
   rp.w1 = (float)p.w1;
   rp.w2 = (float)p.w2;
@@ -164,11 +157,23 @@ extern "C" eat_status eat_route_noalloc(const void* x, int32_t T, int32_t d_mode
   rp.ppl_down = (float)p.ppl_down;
 
   cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = eat::launch_router_logits(x, xdtype == EAT_BF16, w_router, T, d_model,
-                                            n_experts, split, scratch, st);
-  if (e == cudaSuccess)
-    e = eat::launch_route_select(scratch, split, b_router, T, n_experts, p.max_k, N, P, C, rp,
-                                 idx, w, k, nullptr, st);
+  cudaError_t e;
+  if (eat::route_fused(x, xdtype == EAT_BF16, w_router, T, d_model, n_experts)) {
+    e = eat::launch_route_fused(x, xdtype == EAT_BF16, w_router, b_router, T, d_model, n_experts,
+                                p.max_k, N, P, C, rp, idx, w, k, nullptr, st);
+  } else {
+    float2* scratch = nullptr;
+    const eat_status s = scratch_address(&scratch);
+    if (s != EAT_OK) return s;
+
+    int split = eat::router_split(T, d_model, n_experts);
+    while (split > 1 && (size_t)split * T * n_experts > kScratchScores) split /= 2;
+    e = eat::launch_router_logits(x, xdtype == EAT_BF16, w_router, T, d_model, n_experts, split,
+                                  scratch, st);
+    if (e == cudaSuccess)
+      e = eat::launch_route_select(scratch, split, b_router, T, n_experts, p.max_k, N, P, C, rp,
+                                   idx, w, k, nullptr, st);
+  }
   if (e != cudaSuccess) {
     eat::set_thread_error((std::string("eat_route_noalloc launch: ") + cudaGetErrorString(e))
                               .c_str());

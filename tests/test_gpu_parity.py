@@ -303,6 +303,40 @@ def test_router_runs_split_between_blocks(E, d):
     L.close()
 
 
+@pytest.mark.parametrize("dtype,E,d,Ts", [
+    (torch.bfloat16, 64, 2048, (1, 31, 39, 128)),   # one token per cluster; four; the largest
+    (torch.bfloat16, 8, 4096, (1, 19, 20, 512)),    # clusters of eight; last call past 128 tokens
+    (torch.bfloat16, 256, 576, (2, 77)),            # a 64-column second slice, four rounds of experts
+    (torch.bfloat16, 1, 64, (5,)),
+    (torch.bfloat16, 33, 4160, (1, 128)),           # nine slices: the two-kernel path
+    (torch.float32, 100, 640, (3, 300)),            # fp32 hidden states beyond 128 tokens
+])
+def test_small_call_routing(dtype, E, d, Ts):
+    """Scores and selection of small calls in one launch: cluster sizes, ragged slices, ragged token
+    groups and expert rounds against the oracle, from seeded accounts; the same through
+    eat_route_noalloc."""
+    sh = W.scaled(W.OLMOE, f"sr{E}-{d}", d_model=d, n_experts=E, d_ff=64, max_k=min(E, 5),
+                  wdtype=dtype, xdtype=dtype)
+    lw = W.make_layer(sh)
+    ref = oracle_layer(lw)
+    L = eat.EatLayer.from_workload(lw, max(Ts), gpu_params(sh))
+    L.forward(W.make_tokens(sh, Ts[0], step=9).cuda(), 0)  # some history in the accounts
+    N, P, C = L.accounts()
+    acc = orc.Accounts(N.cpu().numpy(), P.cpu().numpy(), C.cpu().numpy())
+    prm = orc.Params(max_k=sh.max_k, temperature=sh.temperature)
+    xdt = eat.EAT_F32 if dtype == torch.float32 else eat.EAT_BF16
+    for T in Ts:
+        x = W.make_tokens(sh, T, step=T).cuda()
+        idx, w, k = L.route(x, 0)
+        routing = orc.route(np64(x), ref, acc, prm, 0)
+        par.check_routing(routing, par.gpu_selection(idx, k), w.cpu().numpy(), sh.max_k)
+        idx2, w2, k2 = torch.empty_like(idx), torch.empty_like(w), torch.empty_like(k)
+        eat.eat_route_noalloc(x, T, d, E, xdt, L._keep[0], L._keep[1], N, P, C, L.params, 0,
+                              idx2, w2, k2)
+        assert torch.equal(idx, idx2) and torch.equal(w, w2) and torch.equal(k, k2)
+    L.close()
+
+
 @pytest.mark.parametrize("E,K,T", [(256, 8, 1500), (64, 2, 1100)])
 def test_sm_pair_small_groups(E, K, T):
     """Calls of >= 1024 tokens run the SM-pair GEMMs; with many experts nearly every group is a
