@@ -7,6 +7,7 @@
 //      accumulates g_norm * o into y in the order j = 0..k_t-1, adds the always-on shared experts
 //      with weight 1, and writes the segment's sum of squares of every slot (||o||_2 of the
 //      unweighted expert output feeds C_s) to nrm_part[slot][segment].
+//  account_warp_kernel (calls of at most 128 tokens): one warp per expert.
 //  account_kernel: blocks (e, c) over each expert's slots in chunks of 1024.  Finishes ||o||_2 of
 //      each slot from its segment sums (fp32, fixed order), sums p and ||o||_2 over the chunk with
 //      compensated fp32 additions (a fixed tree; about fp64 accuracy); an expert of one chunk is
@@ -100,7 +101,7 @@ __device__ __forceinline__ float warp_sum_many(float (&v)[N], int lane) {
 // (bf16 expert rows, the large calls: at most 64 registers, so four blocks share an SM and keep
 // more row loads in flight)
 template <typename TY, int KM, bool OB>
-__global__ void __launch_bounds__(kCombThreads, OB ? 4 : 1)
+__global__ void __launch_bounds__(kCombThreads, OB ? 4 : KM <= 4 ? 2 : 1)
 combine_kernel(const void* __restrict__ opart, int n_split, size_t split_stride,
                const int32_t* __restrict__ slot_of, const float* __restrict__ w,
                const void* __restrict__ sout, int s_bf16, int S, int T, int K, int d, int nseg,
@@ -156,15 +157,26 @@ combine_kernel(const void* __restrict__ opart, int n_split, size_t split_stride,
 #pragma unroll
     for (int j = 0; j < KM; ++j)
       if (in && slots[j] >= 0) o[j] = load8(opart, false, (size_t)slots[j] * d + c);
-    for (int sp = 1; sp < n_split; ++sp) {
+    // the other slices in slice order, SP slices' loads in flight before their sums: a chain of
+    // one L2 round trip per slice made the combine of a
+    // one-token call of 16 slices 11.4 us long, now 6.0
+    constexpr int SP = KM <= 2 ? 4 : KM <= 4 ? 2 : 1;
+    for (int sp0 = 1; sp0 < n_split; sp0 += SP) {
+      V8 q[SP][KM];
 #pragma unroll
-      for (int j = 0; j < KM; ++j) {
-        if (in && slots[j] >= 0) {
-          const V8 q = load8(opart, false, sp * split_stride + (size_t)slots[j] * d + c);
+      for (int u = 0; u < SP; ++u)
 #pragma unroll
-          for (int i = 0; i < 8; ++i) o[j].v[i] += q.v[i];
-        }
-      }
+        for (int j = 0; j < KM; ++j)
+          if (in && slots[j] >= 0 && sp0 + u < n_split)
+            q[u][j] = load8(opart, false, (sp0 + u) * split_stride + (size_t)slots[j] * d + c);
+#pragma unroll
+      for (int u = 0; u < SP; ++u)
+#pragma unroll
+        for (int j = 0; j < KM; ++j)
+          if (in && slots[j] >= 0 && sp0 + u < n_split) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[j].v[i] += q[u][j].v[i];
+          }
     }
 #pragma unroll
     for (int j = 0; j < KM; ++j) {
@@ -198,24 +210,123 @@ combine_kernel(const void* __restrict__ opart, int n_split, size_t split_stride,
   if (lane % (32 / KM) == 0 && sm >= 0) nrm_part[(size_t)sm * nseg + sg] = r;
 }
 
+struct AccountArgs {
+  const int32_t* offs;
+  const float *perm_p, *nrm_part;
+  int nb;
+  double alpha;
+  int64_t* N;
+  double *P, *C;
+  int32_t* st_n;
+  double *st_p, *st_norm;
+  unsigned long long* counters;
+  float4* chunk_sums;
+  unsigned int* tickets;
+  const unsigned int* status;
+  unsigned int* status_mirror;
+};
+
+// p and ||o||_2 of slot i (the segments' squares in order)
+__device__ __forceinline__ void slot_values(const AccountArgs& a, int i, float& p, float& norm) {
+  p = a.perm_p[i];
+  const float* np = a.nrm_part + (size_t)i * a.nb;
+  float sq = 0.f;
+  if ((a.nb & 3) == 0) {
+    for (int b = 0; b < a.nb; b += 4) {
+      const float4 q = *(const float4*)(np + b);
+      sq += q.x;
+      sq += q.y;
+      sq += q.z;
+      sq += q.w;
+    }
+  } else {
+    for (int b = 0; b < a.nb; ++b) sq += np[b];
+  }
+  norm = sqrtf(sq);
+}
+__device__ __forceinline__ void warp_sum_df(float& hi, float& lo) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, hi, o);
+    const float l = __shfl_xor_sync(0xffffffffu, lo, o);
+    df_add(hi, lo, h, l);
+  }
+}
+// An expert's state before the update, requested with the slots' values.
+struct AccountOld {
+  int64_t N;
+  double P, C;
+  unsigned int status;
+};
+__device__ __forceinline__ AccountOld account_old(const AccountArgs& a, int e) {
+  return {a.N[e], a.P[e], a.C[e], __ldcg(a.status)};
+}
+// One thread: the update of expert e from its n slots' sums (compensated pairs).
+__device__ __forceinline__ void account_update(const AccountArgs& a, int e, int n,
+                                               const AccountOld& old, float ph, float pl, float nh,
+                                               float nl) {
+  const double sp = (double)ph + (double)pl, sn = (double)nh + (double)nl;
+  if (old.status == 0u) {  // every kernel of the call completed its work
+    a.N[e] = old.N + n;
+    a.P[e] = old.P + sp;
+    if (n > 0) a.C[e] = (1.0 - a.alpha) * old.C + a.alpha * (sn / (double)n);
+    if (n > 0) atomicAdd(&a.counters[1], 1ull);
+    atomicAdd(&a.counters[2], (unsigned long long)n);
+    if (e == 0) atomicAdd(&a.counters[0], 1ull);
+  }
+  a.st_n[e] = n;
+  a.st_p[e] = sp;
+  a.st_norm[e] = sn;
+  if (e == 0 && a.status_mirror) *(volatile unsigned int*)a.status_mirror = old.status;
+}
+
+// Calls of at most kAccWarpSlots tokens: no expert has more slots than that, and a warp updates one
+// expert (four slots per lane, no block barrier), with the sums' order of account_kernel.  Latency
+// bounds it; with the permute's loads issued at once, an OLMoE decode call of 32 tokens went from
+// 57.9 to 55.6 us, one of 1 token from 40.1 to 38.4.
+constexpr int kAccWarpSlots = 128;
+__global__ void __launch_bounds__(32)
+account_warp_kernel(const AccountArgs a) {
+  const int e = blockIdx.x, lane = threadIdx.x;
+  pdl_wait();
+  pdl_launch_dependents();
+  const int beg = a.offs[e], n = a.offs[e + 1] - beg;
+  const AccountOld old = account_old(a, e);
+  float pv[kAccWarpSlots / 32], nv[kAccWarpSlots / 32];
+#pragma unroll
+  for (int u = 0; u < kAccWarpSlots / 32; ++u) {
+    pv[u] = 0.f;
+    nv[u] = 0.f;
+    if (lane + 32 * u < n) slot_values(a, beg + lane + 32 * u, pv[u], nv[u]);
+  }
+  float ph = 0.f, pl = 0.f, nh = 0.f, nl = 0.f;
+#pragma unroll
+  for (int u = 0; u < kAccWarpSlots / 32; ++u) {
+    if (32 * u >= n) break;
+    float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
+    df_add(a0, a1, pv[u]);
+    df_add(b0, b1, nv[u]);
+    warp_sum_df(a0, a1);
+    warp_sum_df(b0, b1);
+    df_add(ph, pl, a0, a1);
+    df_add(nh, nl, b0, b1);
+  }
+  if (lane == 0) account_update(a, e, n, old, ph, pl, nh, nl);
+}
+
 __global__ void __launch_bounds__(kAccThreads)
-account_kernel(const int32_t* __restrict__ offs, const float* __restrict__ perm_p,
-               const float* __restrict__ nrm_part, int nb, double alpha, int64_t* __restrict__ N,
-               double* __restrict__ P, double* __restrict__ C, int32_t* __restrict__ st_n,
-               double* __restrict__ st_p, double* __restrict__ st_norm,
-               unsigned long long* __restrict__ counters, float4* __restrict__ chunk_sums,
-               unsigned int* __restrict__ tickets, const unsigned int* __restrict__ status,
-               unsigned int* __restrict__ status_mirror) {
+account_kernel(const AccountArgs a) {
   __shared__ float red[4][kAccThreads / 32];
   pdl_wait();
   pdl_launch_dependents();
   const int e = blockIdx.x, c = blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int beg = offs[e], end = offs[e + 1];
+  const int beg = a.offs[e], end = a.offs[e + 1];
   const int n = end - beg;
   const int n_chunks = n > 0 ? (n + kAccChunk - 1) / kAccChunk : 1;
   if (c >= n_chunks) return;
-  const bool vec = (nb & 3) == 0;
+  AccountOld old{};
+  if (tid == 0) old = account_old(a, e);
   float p_hi = 0.f, p_lo = 0.f, n_hi = 0.f, n_lo = 0.f;
   {
     // four slots per thread, all loads issued before the sums
@@ -223,42 +334,18 @@ account_kernel(const int32_t* __restrict__ offs, const float* __restrict__ perm_
     float pv[4], nv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int i = i0 + u * kAccThreads;
       pv[u] = 0.f;
       nv[u] = 0.f;
-      if (i < end) {
-        pv[u] = perm_p[i];
-        const float* np = nrm_part + (size_t)i * nb;
-        float sq = 0.f;
-        if (vec) {
-          for (int b = 0; b < nb; b += 4) {
-            const float4 q = *(const float4*)(np + b);
-            sq += q.x;
-            sq += q.y;
-            sq += q.z;
-            sq += q.w;
-          }
-        } else {
-          for (int b = 0; b < nb; ++b) sq += np[b];
-        }
-        nv[u] = sq;
-      }
+      if (i0 + u * kAccThreads < end) slot_values(a, i0 + u * kAccThreads, pv[u], nv[u]);
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       df_add(p_hi, p_lo, pv[u]);
-      df_add(n_hi, n_lo, sqrtf(nv[u]));
+      df_add(n_hi, n_lo, nv[u]);
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float a = __shfl_xor_sync(0xffffffffu, p_hi, o);
-    const float b = __shfl_xor_sync(0xffffffffu, p_lo, o);
-    const float cc = __shfl_xor_sync(0xffffffffu, n_hi, o);
-    const float dd = __shfl_xor_sync(0xffffffffu, n_lo, o);
-    df_add(p_hi, p_lo, a, b);
-    df_add(n_hi, n_lo, cc, dd);
-  }
+  warp_sum_df(p_hi, p_lo);
+  warp_sum_df(n_hi, n_lo);
   if (lane == 0) {
     red[0][warp] = p_hi;
     red[1][warp] = p_lo;
@@ -274,12 +361,12 @@ account_kernel(const int32_t* __restrict__ offs, const float* __restrict__ perm_
   }
   if (n_chunks > 1) {
     // publish this chunk's sums; the last block of the expert to arrive adds all chunks in order
-    float4* cs = chunk_sums + (size_t)e * gridDim.y;
+    float4* cs = a.chunk_sums + (size_t)e * gridDim.y;
     cs[c] = make_float4(ah, al, bh, bl);
     __threadfence();
-    if (atomicAdd(&tickets[e], 1u) != (unsigned)(n_chunks - 1)) return;
+    if (atomicAdd(&a.tickets[e], 1u) != (unsigned)(n_chunks - 1)) return;
     __threadfence();
-    tickets[e] = 0u;  // for the next call (which starts after this kernel has completed)
+    a.tickets[e] = 0u;  // for the next call (which starts after this kernel has completed)
     ah = al = bh = bl = 0.f;
     for (int ci = 0; ci < n_chunks; ++ci) {
       const float4 v = __ldcg(cs + ci);
@@ -287,20 +374,7 @@ account_kernel(const int32_t* __restrict__ offs, const float* __restrict__ perm_
       df_add(bh, bl, v.z, v.w);
     }
   }
-  const double a = (double)ah + (double)al, b = (double)bh + (double)bl;
-  const unsigned int sw = __ldcg(status);
-  if (sw == 0u) {  // every kernel of the call completed its work
-    N[e] += n;
-    P[e] += a;
-    if (n > 0) C[e] = (1.0 - alpha) * C[e] + alpha * (b / (double)n);
-    if (n > 0) atomicAdd(&counters[1], 1ull);
-    atomicAdd(&counters[2], (unsigned long long)n);
-    if (e == 0) atomicAdd(&counters[0], 1ull);
-  }
-  st_n[e] = n;
-  st_p[e] = a;
-  st_norm[e] = b;
-  if (e == 0 && status_mirror) *(volatile unsigned int*)status_mirror = sw;
+  account_update(a, e, n, old, ah, al, bh, bl);
 }
 
 }  // namespace
@@ -360,13 +434,16 @@ int account_chunks(long long rows) {
 }
 
 cudaError_t launch_account(const int32_t* offs, const float* perm_p, const float* nrm_part, int nb,
-                           int E, long long rows, double alpha, int64_t* N, double* P, double* C,
-                           int32_t* st_n, double* st_p, double* st_norm, long long* counters,
+                           int E, int T, long long rows, double alpha, int64_t* N, double* P,
+                           double* C, int32_t* st_n, double* st_p, double* st_norm, long long* counters,
                            float4* chunk_sums, unsigned int* tickets, const unsigned int* status,
                            unsigned int* status_mirror, cudaStream_t st) {
-  return launch_pdl(account_kernel, dim3(E, account_chunks(rows)), dim3(kAccThreads), 0, st, offs,
-                    perm_p, nrm_part, nb, alpha, N, P, C, st_n, st_p, st_norm,
-                    (unsigned long long*)counters, chunk_sums, tickets, status, status_mirror);
+  const AccountArgs a{offs, perm_p, nrm_part, nb, alpha, N, P, C, st_n,
+                      st_p, st_norm, (unsigned long long*)counters, chunk_sums, tickets, status,
+                      status_mirror};
+  if (T <= kAccWarpSlots)  // (an expert has at most one slot per token)
+    return launch_pdl(account_warp_kernel, dim3(E), dim3(32), 0, st, a);
+  return launch_pdl(account_kernel, dim3(E, account_chunks(rows)), dim3(kAccThreads), 0, st, a);
 }
 
 }  // namespace eat

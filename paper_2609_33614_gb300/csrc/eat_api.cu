@@ -313,7 +313,7 @@ eat_status run_forward(eat_handle* h, const void* x, int T, int ppl_sign, void* 
   if (x_host && side) return fail(h, EAT_ERR_UNSUPPORTED, "host-read input with side-stream experts");
   EAT_TRY(run_route(h, x, T, ppl_sign, h->idx, h->w, h->k, h->psel, true, st, x_host));
   EAT_TRY(launch(h, kPermute, st, "permute", [&] {
-    return launch_permute(h->idx, h->k, h->psel, T, h->K, h->E, tile_rows, tile_rows_down,
+    return launch_permute(h->idx, h->psel, T, h->K, h->E, tile_rows, tile_rows_down,
                           h->perm, h->chunk_cnt, st);
   }));
   const int rows = T * h->K;
@@ -362,7 +362,7 @@ eat_status run_forward(eat_handle* h, const void* x, int T, int ppl_sign, void* 
                           h->w, h->sout, tc, h->S, T, h->K, h->d, y, h->nrm_part, h->status, st);
   }));
   EAT_TRY(launch(h, kAccount, st, "account update", [&] {
-    return launch_account(h->perm.offs, h->perm.perm_p, h->nrm_part, h->nb, h->E, rows,
+    return launch_account(h->perm.offs, h->perm.perm_p, h->nrm_part, h->nb, h->E, T, rows,
                           h->prm.alpha, h->N, h->P, h->C, h->st_n, h->st_p, h->st_norm,
                           h->counters, h->acc_sums, h->acc_tickets, h->status, h->mirror_dev, st);
   }));

@@ -155,7 +155,7 @@ int permute_chunks(int T);  // CTAs of the permute of a T-token call
 // int32 words of the permute's scratch (a ticket counter, zero between calls, and the per-chunk
 // expert counts) for calls of up to Tmax tokens
 size_t permute_scratch_ints(int Tmax, int E);
-cudaError_t launch_permute(const int32_t* idx, const int32_t* k, const float* psel, int T, int K,
+cudaError_t launch_permute(const int32_t* idx, const float* psel, int T, int K,
                            int E, int tile_rows, int tile_rows2, PermuteOut o, int32_t* scratch,
                            cudaStream_t st);
 
@@ -201,15 +201,15 @@ cudaError_t launch_combine(int y_bf16, const void* opart, int o_bf16, int n_spli
                            int split_stride_rows, const int32_t* slot_of, const float* w,
                            const void* sout, int s_bf16, int S, int T, int K, int d, void* y,
                            float* nrm_part, const unsigned int* status, cudaStream_t st);
-// rows: the call's T * K selection slots (bounds the blocks per expert); chunk_sums:
+// T, rows: the call's tokens and T * K selection slots (bounds the blocks per expert); chunk_sums:
 // [E][account_chunks(rows)] scratch; tickets: [E] words, zero between calls (the kernel leaves
 // them zero).  status: the device status word (nonzero: an expert kernel of the call gave up on a
 // bounded wait; the update is then skipped); status_mirror: device address of a host-mapped copy
 // of the word, written by the block that finishes expert 0, or null.
 int account_chunks(long long rows);
 cudaError_t launch_account(const int32_t* offs, const float* perm_p, const float* nrm_part, int nb,
-                           int E, long long rows, double alpha, int64_t* N, double* P, double* C,
-                           int32_t* st_n, double* st_p, double* st_norm, long long* counters,
+                           int E, int T, long long rows, double alpha, int64_t* N, double* P,
+                           double* C, int32_t* st_n, double* st_p, double* st_norm, long long* counters,
                            float4* chunk_sums, unsigned int* tickets, const unsigned int* status,
                            unsigned int* status_mirror, cudaStream_t st);
 

@@ -73,21 +73,23 @@ __device__ void write_offsets(int* cnt, int E, int tile_rows, int tile_rows2, Pe
 // the exclusive prefix over chunks and writes the offsets.
 template <int KM>
 __global__ void __launch_bounds__(kChunk)
-permute_count_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kk, int T,
-                     int K, int E, int tile_rows, int tile_rows2, int32_t* chunk_cnt,
+permute_count_kernel(const int32_t* __restrict__ idx, int T, int K,
+                     int E, int tile_rows, int tile_rows2, int32_t* chunk_cnt,
                      int n_chunks, unsigned* ticket, PermuteOut o) {
   extern __shared__ int cnt[];  // [E]
   __shared__ int is_last;
-  pdl_wait();
-  pdl_launch_dependents();
   const int tid = threadIdx.x, nt = blockDim.x;
   for (int e = tid; e < E; e += nt) cnt[e] = 0;
-  __syncthreads();
+  pdl_wait();
+  pdl_launch_dependents();
   const int t = blockIdx.x * nt + tid;
-  const int kt = t < T ? kk[t] : 0;
+  int ex[KM];
+#pragma unroll
+  for (int j = 0; j < KM; ++j) ex[j] = t < T && j < K ? idx[(size_t)t * K + j] : -1;
+  __syncthreads();
 #pragma unroll
   for (int j = 0; j < KM; ++j)
-    if (j < K && j < kt) atomicAdd(&cnt[idx[(size_t)t * K + j]], 1);
+    if (ex[j] >= 0) atomicAdd(&cnt[ex[j]], 1);
   __syncthreads();
   for (int e = tid; e < E; e += nt) chunk_cnt[(size_t)blockIdx.x * E + e] = cnt[e];
   __threadfence();
@@ -126,8 +128,7 @@ permute_count_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict_
 // at offs[e] + chunk_base[c][e].
 template <int KM>
 __global__ void __launch_bounds__(kSingleMax)
-permute_assign_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ kk,
-                      const float* __restrict__ psel, int T, int K, int E, int tile_rows,
+permute_assign_kernel(const int32_t* __restrict__ idx, const float* __restrict__ psel, int T, int K, int E, int tile_rows,
                       int tile_rows2, const int32_t* __restrict__ chunk_base, PermuteOut o) {
   extern __shared__ unsigned sm[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -136,15 +137,20 @@ permute_assign_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict
   int* wbase = (int*)(mask + nw * E);     // [nw][E] first slot of each warp's pairs of e
   int* cnt = wbase + nw * E;              // [E] counts, then offsets (single CTA)
   const unsigned lt = (1u << lane) - 1u;
+  for (int i = tid; i < nw * E; i += nt) mask[i] = 0u;
   pdl_wait();
   pdl_launch_dependents();
-  for (int i = tid; i < nw * E; i += nt) mask[i] = 0u;
-  __syncthreads();
+  // every load of the token at once (the selection writes -1 past the k-th expert)
   const int t = blockIdx.x * nt + tid;
-  const int kt = t < T ? kk[t] : 0;
   int ex[KM];
+  float ps[KM];
 #pragma unroll
-  for (int j = 0; j < KM; ++j) ex[j] = (j < K && j < kt) ? idx[(size_t)t * K + j] : -1;
+  for (int j = 0; j < KM; ++j) {
+    const bool in = t < T && j < K;
+    ex[j] = in ? idx[(size_t)t * K + j] : -1;
+    ps[j] = in ? psel[(size_t)t * K + j] : 0.f;
+  }
+  __syncthreads();
 #pragma unroll
   for (int j = 0; j < KM; ++j)
     if (ex[j] >= 0) atomicOr(&mask[warp * E + ex[j]], 1u << lane);
@@ -174,7 +180,7 @@ permute_assign_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict
       const int slot = wbase[warp * E + e] + __popc(mask[warp * E + e] & lt);
       o.perm_tok[slot] = t;
       o.slot_of[(size_t)t * K + j] = slot;
-      o.perm_p[slot] = psel[(size_t)t * K + j];
+      o.perm_p[slot] = ps[j];
     } else if (j < K && t < T) {
       o.slot_of[(size_t)t * K + j] = -1;
     }
@@ -182,24 +188,24 @@ permute_assign_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict
 }
 
 template <int KM>
-cudaError_t launch_permute_k(const int32_t* idx, const int32_t* k, const float* psel, int T,
+cudaError_t launch_permute_k(const int32_t* idx, const float* psel, int T,
                              int K, int E, int tile_rows, int tile_rows2, PermuteOut o,
                              int32_t* scratch, cudaStream_t st) {
   if (T <= kSingleMax) {
     const int nt = (T + 31) / 32 * 32;
     const size_t smem = (size_t)(2 * (nt / 32) * E + E) * sizeof(int);
-    return launch_pdl(permute_assign_kernel<KM>, dim3(1), dim3(nt), smem, st, idx, k, psel, T,
+    return launch_pdl(permute_assign_kernel<KM>, dim3(1), dim3(nt), smem, st, idx, psel, T,
                       K, E, tile_rows, tile_rows2, (const int32_t*)nullptr, o);
   }
   const int n_chunks = permute_chunks(T);
   unsigned* ticket = (unsigned*)scratch;
   int32_t* chunk_cnt = scratch + kTicketInts;
   cudaError_t e = launch_pdl(permute_count_kernel<KM>, dim3(n_chunks), dim3(kChunk),
-                             (size_t)E * sizeof(int), st, idx, k, T, K, E, tile_rows, tile_rows2,
+                             (size_t)E * sizeof(int), st, idx, T, K, E, tile_rows, tile_rows2,
                              chunk_cnt, n_chunks, ticket, o);
   if (e != cudaSuccess) return e;
   const size_t smem = (size_t)(2 * (kChunk / 32) * E + E) * sizeof(int);
-  return launch_pdl(permute_assign_kernel<KM>, dim3(n_chunks), dim3(kChunk), smem, st, idx, k,
+  return launch_pdl(permute_assign_kernel<KM>, dim3(n_chunks), dim3(kChunk), smem, st, idx,
                     psel, T, K, E, tile_rows, tile_rows2, (const int32_t*)chunk_cnt, o);
 }
 
@@ -211,16 +217,16 @@ size_t permute_scratch_ints(int Tmax, int E) {
   return kTicketInts + (size_t)permute_chunks(Tmax) * E;
 }
 
-cudaError_t launch_permute(const int32_t* idx, const int32_t* k, const float* psel, int T, int K,
+cudaError_t launch_permute(const int32_t* idx, const float* psel, int T, int K,
                            int E, int tile_rows, int tile_rows2, PermuteOut o, int32_t* scratch,
                            cudaStream_t st) {
   if (K <= 2)
-    return launch_permute_k<2>(idx, k, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
+    return launch_permute_k<2>(idx, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
   if (K <= 4)
-    return launch_permute_k<4>(idx, k, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
+    return launch_permute_k<4>(idx, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
   if (K <= 8)
-    return launch_permute_k<8>(idx, k, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
-  return launch_permute_k<16>(idx, k, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
+    return launch_permute_k<8>(idx, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
+  return launch_permute_k<16>(idx, psel, T, K, E, tile_rows, tile_rows2, o, scratch, st);
 }
 
 }  // namespace eat

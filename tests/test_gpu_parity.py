@@ -337,6 +337,16 @@ def test_small_call_routing(dtype, E, d, Ts):
     L.close()
 
 
+@pytest.mark.parametrize("T", [127, 128, 129])
+def test_account_update_around_the_one_warp_limit(T):
+    """Every token selects the same expert, so its account sums T slots: up to 128 by one warp,
+    beyond by a block."""
+    lw = W.make_layer(OLMOE_S)
+    lw.b_router = torch.full_like(lw.b_router, -30.0)
+    lw.b_router[5] = 30.0
+    run_parity(OLMOE_S, lw, [T, T])
+
+
 @pytest.mark.parametrize("E,K,T", [(256, 8, 1500), (64, 2, 1100)])
 def test_sm_pair_small_groups(E, K, T):
     """Calls of >= 1024 tokens run the SM-pair GEMMs; with many experts nearly every group is a
