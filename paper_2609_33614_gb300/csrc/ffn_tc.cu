@@ -5,7 +5,7 @@
 //
 // Orientation ("swap AB"): a tile is 128 weight rows (output features of one expert) x BN tokens
 // (16..128 rows of that expert's slot list), so decode calls with a handful of tokens still issue
-// full M = 128 MMAs and simply stream the activated experts' weights.  Calls of 1024 tokens or more
+// full M = 128 MMAs and simply stream the activated experts' weights.  Calls of 512 tokens or more
 // run on SM pairs instead (tc_pair_kernel below: M = 256 weight rows x 256 tokens per MMA).
 //   gate/up kernel: D_gate = Wg[e, f0:f0+128, :] . Xperm[slots]^T and D_up likewise, both in TMEM;
 //       the epilogue writes act[slot, f] = silu(D_gate) * D_up in bf16 (fp32 accumulation).
@@ -1446,16 +1446,21 @@ cudaError_t launch_down_bn(int bn, const CUtensorMap& a0, const CUtensorMap& b,
 }  // namespace
 
 // The largest group of a call has at most T rows (each token picks an expert once).  Calls of at
-// least kPairMinTokens run both expert GEMMs on SM pairs with 256-token tiles (interleaved gate/
-// up, 256-feature down tiles); smaller calls use single-SM kernels with tiles of the smallest
-// width that holds T, at most 128.  (On a single SM the interleaved 256-token gate/up moves the
-// same shared-memory bytes per flop as two 128-token accumulators and measured slower: OLMoE
-// prefill gate/up 294 -> 316 us.)
-constexpr int kPairMinTokens = 1024;
+// least kPairMinTokens tokens, or with kPairMinRows per expert on average, run both expert GEMMs on
+// SM pairs with 256-token tiles (interleaved gate/up, 256-feature down tiles); smaller calls use
+// single-SM kernels with tiles of the smallest width that holds T, at most 128.  us per call, single
+// SM / pairs: Mixtral shape 200 tokens (50 rows per expert) 482 / 476, 400 618 / 536, 1000 978 /
+// 785; OLMoE 333 (41) 131 / 151, 600 (75) 159 / 159, 1000 205 / 194; Qwen 600 (40) 192 / 177, 1000
+// 234 / 203; DeepSeek-V2-Lite 333 (31) 209 / 223, 600 (56) 231 / 233, 1000 300 / 265.  (On a single
+// SM the interleaved 256-token gate/up moves the same shared-memory bytes per flop as two 128-token
+// accumulators and measured slower: OLMoE prefill gate/up 294 -> 316 us.)
+constexpr int kPairMinTokens = 512, kPairMinRows = 64;
 int tc_tile_rows(const TcLayer& L, int T) {
   for (int i = 0; i < kNumBN - 1; ++i)
     if (T <= kBNs[i]) return kBNs[i];
-  return T >= kPairMinTokens && !L.w8 ? kPairBN : 128;
+  const bool pair = T >= kPairMinTokens || (T > kBNs[kNumBN - 1] &&
+                                            (long long)T * L.K >= (long long)kPairMinRows * L.E);
+  return pair && !L.w8 ? kPairBN : kBNs[kNumBN - 1];
 }
 // Small calls gather their token rows inside the gate/up kernel (one launch and one HBM round
 // trip fewer); large calls copy them to Xperm first: there the shared-memory-bound gate/up kernel

@@ -357,6 +357,16 @@ def test_sm_pair_small_groups(E, K, T):
     run_parity(sh, lw, [T, T])
 
 
+@pytest.mark.parametrize("E,K,S,T", [(64, 4, 2, 512), (8, 2, 0, 256), (5, 5, 0, 129)])
+def test_sm_pair_smallest_calls(E, K, S, T):
+    """The smallest calls that run on SM pairs (512 tokens, or 64 rows per expert above 128 tokens):
+    mostly partial tiles, shared experts in the same launches, down projections still split along
+    K; and one token less, on single SMs."""
+    sh = W.scaled(W.QWEN if S else W.OLMOE, f"pairmin{E}", d_model=256, n_experts=E, d_ff=1024,
+                  max_k=K, n_shared=S, d_ff_shared=256 if S else 0)
+    run_parity(sh, W.make_layer(sh), [T, T - 1])
+
+
 def test_sm_pair_one_large_group():
     """One expert takes every token of a 2100-token call: 8 full SM-pair tiles and a partial one."""
     lw = W.make_layer(OLMOE_S)
