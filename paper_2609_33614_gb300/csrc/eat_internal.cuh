@@ -213,6 +213,10 @@ cudaError_t launch_account(const int32_t* offs, const float* perm_p, const float
                            float4* chunk_sums, unsigned int* tickets, const unsigned int* status,
                            unsigned int* status_mirror, cudaStream_t st);
 
+// Copies the accounts to the caller's [E] arrays.
+cudaError_t launch_read_accounts(const int64_t* N, const double* P, const double* C, int E,
+                                 int64_t* outN, double* outP, double* outC, cudaStream_t st);
+
 // §3.3 perplexity of a window of token negative log-likelihoods and the sign of its change.
 cudaError_t launch_ppl_update(const float* nll, int n, double* state, int32_t* sign,
                               cudaStream_t st);

@@ -337,6 +337,48 @@ def test_small_call_routing(dtype, E, d, Ts):
     L.close()
 
 
+@pytest.mark.parametrize("which", ["all", "some", "misaligned"])
+def test_routing_and_account_outputs(which):
+    """The caller's routing buffers, all, some or (misaligned) copied at the end, hold what eat_route
+    gives for the same accounts, and the call's other results do not depend on them; accounts read
+    into aligned and misaligned arrays."""
+    lw = W.make_layer(OLMOE_S)
+    T, K, E = 40, OLMOE_S.max_k, OLMOE_S.n_experts
+    x = W.make_tokens(OLMOE_S, T).cuda()
+    A, B = (eat.EatLayer.from_workload(lw, T, gpu_params(OLMOE_S)) for _ in range(2))
+    idx0, w0, k0 = A.route(x, 0)
+    y0 = A.forward(x, 0)
+    off = 1 if which == "misaligned" else 0  # bytes
+
+    def buf(n):
+        raw = torch.zeros(4 * n + 16, dtype=torch.uint8, device="cuda")
+        return raw, raw.data_ptr() + off
+    bi, bw, bk = buf(T * K), buf(T * K), buf(T)
+    y = torch.empty_like(x)
+    some = which == "some"
+    eat._check(eat.lib().eat_moe_forward(B.h, x.data_ptr(), T, 0, y.data_ptr(), bi[1],
+                                         None if some else bw[1], None if some else bk[1],
+                                         torch.cuda.current_stream().cuda_stream), B.h)
+    torch.cuda.synchronize()
+
+    def read(b, n, dt):
+        return b[0][off:off + 4 * n].clone().view(dt)
+    assert torch.equal(y, y0)
+    assert torch.equal(read(bi, T * K, torch.int32).view(T, K), idx0)
+    if not some:
+        assert torch.equal(read(bw, T * K, torch.float32).view(T, K), w0)
+        assert torch.equal(read(bk, T, torch.int32), k0)
+    ref = A.accounts()
+    raws = [torch.zeros(8 * E + 16, dtype=torch.uint8, device="cuda") for _ in range(3)]
+    eat._check(eat.lib().eat_get_accounts(B.h, *[r.data_ptr() + off for r in raws],
+                                          torch.cuda.current_stream().cuda_stream), B.h)
+    torch.cuda.synchronize()
+    for r, want in zip(raws, ref):
+        assert torch.equal(r[off:off + 8 * E].clone().view(want.dtype), want)
+    A.close()
+    B.close()
+
+
 @pytest.mark.parametrize("T", [127, 128, 129])
 def test_account_update_around_the_one_warp_limit(T):
     """Every token selects the same expert, so its account sums T slots: up to 128 by one warp,
