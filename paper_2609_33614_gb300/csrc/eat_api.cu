@@ -334,7 +334,7 @@ eat_status run_forward(eat_handle* h, const void* x, int T, int ppl_sign, void* 
     };
     if (h->w8)
       EAT_TRY(split(TcSplit::kSlotX, "split x (slots)"));
-    else if (!tc_gathers_in_kernel(h->tc, T))
+    else if (!tc_token_tiles(h->tc, T))
       EAT_TRY(launch(h, kGather, st, "gather rows",
                      [&] { return tc_launch_gather(h->tc, c, st); }));
     EAT_TRY(launch(h, kUp, st, "tc gate/up", [&] { return tc_launch_up(h->tc, c, false, st); }));

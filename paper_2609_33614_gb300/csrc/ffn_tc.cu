@@ -141,11 +141,6 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-// The proxy fence that orders bytes copied by cp.async (generic proxy) before the tensor core
-// reads them (async proxy).
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -252,7 +247,7 @@ struct Cfg {
   static constexpr int kKPS = 6 * kSubBytes <= kSmemBudget - 2048 ? 2 : 1;
   // e4m3 tiles of 64 or more tokens are drained by two warps per TMEM lane quarter (one per half
   // of the tile's columns), so an accumulator buffer returns to the MMA issuer sooner (e4m3
-  // prefill +20 %; the bf16 gathering gate/up at 128-token tiles was slower with eight)
+  // prefill +20 %)
   static constexpr int kEpiWarps = (W8 && BN >= 64) ? 8 : 4;
   static constexpr int kThreads = 64 + 32 * kEpiWarps;
   static constexpr int kStageBytes = kKPS * kSubBytes;
@@ -285,8 +280,8 @@ struct TcArgs {
   void* out;
   long long split_stride;    // elements between split slices of the fp32 output
   int out_bf16;              // down kernel without split-K: write bf16 rows instead of fp32
-  const int32_t* b_rows;     // gather mode: slot -> token; B rows are copied from bx by the warp
-  const __nv_bfloat16* bx;   // gather mode: token rows [T, row stride kblocks * 64] (16-bit)
+  const int32_t* slot_tok;   // token tiles: slot -> token
+  int n_tok;                 // token tiles: tokens of the call
   const float* scale0;       // fp8 weights: per-row scales of the A matrix (gate, or down)
   const float* scale1;       // fp8 weights: per-row scales of the up matrix
   const float* bscale;       // fp8: per-row scales of the B operand, indexed like its rows
@@ -381,13 +376,22 @@ __device__ __forceinline__ float silu_f(float g) { return __fdividef(g, 1.0f + _
 // written by split_e4m3_kernel); a k-block holds the e4m3 A tiles of 128 elements and the hi and
 // lo B tiles, every k-step issues W . hi and W . lo into the same fp32 accumulator
 // (kind::f8f6f4), and the epilogue multiplies by the weight row's scale and the B row's scale.
-template <int BN, int MODE, bool W8>
+//
+// TOK (bf16 gate/up of calls whose tokens fit one tile): the B tile is the call's token rows
+// themselves, in token order, the same for every expert, so TMA loads it from x and no row is
+// gathered; the MMA computes all tokens and the epilogue keeps the columns of those that selected
+// the expert.  A warp that gathered an expert's rows with cp.async was the pace of the launch from
+// 64-token tiles on: OLMoE 48 tokens 76.2 -> 70.7 us per call, 100 93.9 -> 85.9, Qwen 100 86.4 ->
+// 80.7, DeepSeek-V2-Lite 128 172.4 -> 169.2, at most 32 tokens 0.3-1 % less.  (e4m3 layers, whose
+// rows are split into planes anyway, measured 0-3 % slower with it.)
+template <int BN, int MODE, bool W8, bool TOK>
 __global__ void __launch_bounds__(Cfg<BN, MODE, W8>::kThreads, 1)
 tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
               const __grid_constant__ CUtensorMap mapB, const TcArgs args) {
   using C = Cfg<BN, MODE, W8>;
   constexpr bool GATEUP = C::kGateUp;
   constexpr int S = C::kStages;
+  static_assert(!TOK || (GATEUP && !W8), "token tiles are a layout of the bf16 gate/up");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint64_t* full = (uint64_t*)(smem + S * C::kStageBytes);
@@ -401,7 +405,7 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(&full[s], args.b_rows ? 2 : 1);  // + the gathered rows' arrival
+      mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -446,7 +450,7 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
   // start after its own wait): the producer fills the first stages' A tiles while the previous
   // kernel finishes; the B tiles of those stages follow after the wait.
   int pre = 0;  // stages whose A tiles are in flight
-  const bool early = args.prefetch_a && !args.b_rows;  // (gathering launches follow the permute)
+  const bool early = args.prefetch_a;
   if (early) {
     go = stage_offsets(args, s_row, s_tile);
     __syncthreads();
@@ -475,87 +479,7 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
   }
   const int units = count_units();
 
-  if (GATEUP && !W8 && warp == 0 && args.b_rows) {
-    // ------------------------------------------------------------ producer, gathered tokens:
-    // lane 0 issues the weight TMA; all lanes copy the tile's token rows from x with 16-byte
-    // cp.async into the 128B-swizzled B tile of each k-block of the stage (lane l: column chunk
-    // l % 8 of rows l / 8 + 4 i).  A stage's rows are released LAG stages later: wait for the
-    // lane's own copies, fence the async proxy, and one arrive per warp on the stage's full
-    // barrier.
-    constexpr int PER = BN / 4;
-    constexpr int LAG = S > 2 ? S - 2 : 1;
-    const unsigned fullmask = 0xffffffffu;
-    const int cc = lane & 7, r0 = lane >> 3;
-    const size_t ld = (size_t)args.kblocks * kBK;
-    int stage = 0;
-    uint32_t phase = 0;
-    long long it = 0, released = 0;
-    bool ok = true;
-    UnitIter<BN> it_u(units, go);
-    for (Unit w; ok && it_u.next(args, w);) {
-      const int a_row = w.g * args.a_rows_per_group + w.m0;
-      int tok[PER];
-#pragma unroll
-      for (int i = 0; i < PER; ++i) {
-        const int r = r0 + 4 * i;
-        tok[i] = r < w.nrows ? args.b_rows[w.slot0 + r] : -1;
-      }
-      for (int kb = w.kb0; kb < w.kb1; kb += C::kKPS) {
-        const int nk = C::kKPS == 1 ? 1 : min(C::kKPS, w.kb1 - kb);  // k-blocks of this stage
-        bool okw = true;
-        if (lane == 0) okw = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, args.err, 1u, true);
-        okw = __shfl_sync(fullmask, okw ? 1 : 0, 0) != 0;
-        if (!okw) {
-          ok = false;
-          break;
-        }
-        uint8_t* st = smem + stage * C::kStageBytes;
-        if (elect_one()) {
-          mbar_expect_tx(&full[stage], nk * C::kNA * C::kABytes);
-#pragma unroll
-          for (int j = 0; j < C::kKPS; ++j)
-            if (j < nk) load_a(st + j * C::kSubBytes, &full[stage], kb + j, a_row);
-        }
-#pragma unroll
-        for (int j = 0; j < C::kKPS; ++j) {
-          if (j >= nk) break;
-          const uint32_t sb = smem_u32(st + j * C::kSubBytes + C::kNA * C::kABytes);
-#pragma unroll
-          for (int i = 0; i < PER; ++i) {
-            if (tok[i] >= 0) {
-              const int r = r0 + 4 * i;
-              cp_async16(sb + r * 128 + ((cc ^ (r & 7)) << 4),
-                         args.bx + (size_t)tok[i] * ld + (kb + j) * kBK + cc * 8);
-            }
-          }
-        }
-        cp_async_commit();
-        ++it;
-        if (it - released > LAG) {
-          cp_async_wait<LAG>();
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&full[released % S]);
-          ++released;
-        }
-        if (++stage == S) {
-          stage = 0;
-          phase ^= 1u;
-        }
-      }
-    }
-    // release the stages still held (also on abort, so their barriers can complete), then let the
-    // weight copies in flight land before the CTA may exit
-    cp_async_wait<0>();
-    fence_proxy_async();
-    __syncwarp();
-    if (lane == 0) {
-      for (; released < it; ++released) mbar_arrive(&full[released % S]);
-      const long long first = it > S ? it - S : 0;
-      for (long long i = first; i < it; ++i)
-        mbar_wait(&full[i % S], (uint32_t)((i / S) & 1), abort_flag, args.err, 2u, false);
-    }
-  } else if (warp == 0) {
+  if (warp == 0) {
     if (elect_one()) {
       // ------------------------------------------------------------ TMA producer
       int stage = 0;
@@ -565,7 +489,7 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
       UnitIter<BN> it_u(units, go);
       for (Unit w; ok && it_u.next(args, w);) {
         const int a_row = w.g * args.a_rows_per_group + w.m0;
-        const int b_row = w.slot0 - w.g * args.b_shift_per_group;
+        const int b_row = TOK ? 0 : w.slot0 - w.g * args.b_shift_per_group;
         for (int kb = w.kb0; kb < w.kb1; kb += C::kKPS) {
           const int nk = min(C::kKPS, w.kb1 - kb);
           uint8_t* st = smem + stage * C::kStageBytes;
@@ -615,7 +539,7 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
         const uint32_t d1 = d0 + C::kProjCols;
         // MMA width: the tile's rows rounded up to 16 (a partial tile computes no padding; the
         // fused fp8 MMA spans the hi tile's BN rows and the lo tile's first n)
-        const int n_mma = min(BN, (w.nrows + 15) & ~15);
+        const int n_mma = min(BN, ((TOK ? args.n_tok : w.nrows) + 15) & ~15);
         const uint32_t idesc = !W8       ? idesc_bf16(n_mma)
                                : C::kFuse ? idesc_e4m3(BN + n_mma)
                                           : idesc_e4m3(n_mma);
@@ -675,9 +599,21 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
     const int row = 32 * q + lane;
     constexpr int kCols = BN / (C::kEpiWarps / 4);  // the tile columns of one warp
     const int cbeg = ((warp - 2) >> 2) * kCols;
+    __shared__ int32_t s_map[TOK ? C::kEpiWarps : 1][TOK ? kCols : 1];
+    int32_t* map = s_map[TOK ? warp - 2 : 0];  // the slot of each of the warp's tokens, or -1
     int local = 0;
     UnitIter<BN> it_u(units, go);
     for (Unit w; it_u.next(args, w); ++local) {
+      if constexpr (TOK) {
+        __syncwarp();
+        for (int c = lane; c < kCols; c += 32) map[c] = -1;
+        __syncwarp();
+        for (int i = lane; i < w.nrows; i += 32) {
+          const int t = __ldcg(args.slot_tok + w.slot0 + i) - cbeg;
+          if (t >= 0 && t < kCols) map[t] = w.slot0 + i;
+        }
+        __syncwarp();
+      }
       const int buf = local & 1;
       const uint32_t tph = (uint32_t)((local >> 1) & 1);
       if (!warp_wait(&tfull[buf], tph, abort_flag, args.err, 32u)) break;
@@ -692,8 +628,9 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
         if (GATEUP) s1 = args.scale1[ar];
       }
       const float* bsc = W8 ? args.bscale + (w.slot0 - w.g * args.b_shift_per_group) : nullptr;
-      const int cend = min(cbeg + kCols, w.nrows);
+      const int cend = min(cbeg + kCols, TOK ? args.n_tok : w.nrows);
       for (int c0 = cbeg; c0 < cend; c0 += 16) {
+        if (TOK && !__any_sync(0xffffffffu, map[c0 - cbeg + (lane & 15)] >= 0)) continue;
         uint32_t g[16], up[16];
         tmem_ld16(tbase + c0, g);
         if (GATEUP) tmem_ld16(tbase + C::kProjCols + c0, up);
@@ -712,8 +649,9 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
         if (fok) {
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
-            if (c0 + c < w.nrows) {
-              const size_t slot = (size_t)(w.slot0 + c0 + c);
+            const int sl = TOK ? map[c0 - cbeg + c] : w.slot0 + c0 + c;
+            if (TOK ? sl >= 0 : c0 + c < w.nrows) {
+              const size_t slot = (size_t)sl;
               const float sc = W8 ? bsc[c0 + c] : 1.0f;
               const float gv = W8 ? __uint_as_float(g[c]) * (s0 * sc) : __uint_as_float(g[c]);
               if (GATEUP) {
@@ -1347,19 +1285,19 @@ int bn_index(int bn) {
   return kNumBN - 1;
 }
 
-template <int BN, int MODE, bool W8>
+template <int BN, int MODE, bool W8, bool TOK>
 cudaError_t launch_tc(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
                       const TcArgs& args, int grid, cudaStream_t st) {
   using C = Cfg<BN, MODE, W8>;
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(tc_ffn_kernel<BN, MODE, W8>,
+    attr_err = cudaFuncSetAttribute(tc_ffn_kernel<BN, MODE, W8, TOK>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   });
   if (attr_err != cudaSuccess) return attr_err;
   if (grid <= 0) return cudaSuccess;
-  return launch_pdl(tc_ffn_kernel<BN, MODE, W8>, dim3(grid), dim3(C::kThreads), C::kSmemBytes,
+  return launch_pdl(tc_ffn_kernel<BN, MODE, W8, TOK>, dim3(grid), dim3(C::kThreads), C::kSmemBytes,
                     st, a0, a1, b, args);
 }
 
@@ -1421,25 +1359,14 @@ cudaError_t launch_pair(const CUtensorMap& a0, const CUtensorMap& a1, const CUte
 
 // Single-SM launches: token tiles of 16..128 rows (256-row tiles run on SM pairs); W8 for fp8
 // weights (single-SM kernels only, at any call size).
-template <bool W8>
-cudaError_t launch_up_bn(int bn, const CUtensorMap& a0, const CUtensorMap& a1,
-                         const CUtensorMap& b, const TcArgs& args, int grid, cudaStream_t st) {
+template <int MODE, bool W8, bool TOK>
+cudaError_t launch_bn(int bn, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
+                      const TcArgs& args, int grid, cudaStream_t st) {
   switch (bn) {
-    case 16: return launch_tc<16, kModeGateUp, W8>(a0, a1, b, args, grid, st);
-    case 32: return launch_tc<32, kModeGateUp, W8>(a0, a1, b, args, grid, st);
-    case 64: return launch_tc<64, kModeGateUp, W8>(a0, a1, b, args, grid, st);
-    default: return launch_tc<128, kModeGateUp, W8>(a0, a1, b, args, grid, st);
-  }
-}
-
-template <bool W8>
-cudaError_t launch_down_bn(int bn, const CUtensorMap& a0, const CUtensorMap& b,
-                           const TcArgs& args, int grid, cudaStream_t st) {
-  switch (bn) {
-    case 16: return launch_tc<16, kModeDown, W8>(a0, a0, b, args, grid, st);
-    case 32: return launch_tc<32, kModeDown, W8>(a0, a0, b, args, grid, st);
-    case 64: return launch_tc<64, kModeDown, W8>(a0, a0, b, args, grid, st);
-    default: return launch_tc<128, kModeDown, W8>(a0, a0, b, args, grid, st);
+    case 16: return launch_tc<16, MODE, W8, TOK>(a0, a1, b, args, grid, st);
+    case 32: return launch_tc<32, MODE, W8, TOK>(a0, a1, b, args, grid, st);
+    case 64: return launch_tc<64, MODE, W8, TOK>(a0, a1, b, args, grid, st);
+    default: return launch_tc<128, MODE, W8, TOK>(a0, a1, b, args, grid, st);
   }
 }
 
@@ -1462,11 +1389,10 @@ int tc_tile_rows(const TcLayer& L, int T) {
                                             (long long)T * L.K >= (long long)kPairMinRows * L.E);
   return pair && !L.w8 ? kPairBN : kBNs[kNumBN - 1];
 }
-// Small calls gather their token rows inside the gate/up kernel (one launch and one HBM round
-// trip fewer); large calls copy them to Xperm first: there the shared-memory-bound gate/up kernel
-// loses more to the warp's cp.async traffic than the separate gather costs.  fp8 layers always
-// read their B operand from the e4m3 planes that split_e4m3_kernel writes.
-bool tc_gathers_in_kernel(const TcLayer& L, int T) { return T <= 128 && !L.w8; }
+// bf16 calls whose tokens fit one tile read the token rows themselves as the gate/up kernel's B tile
+// (tc_ffn_kernel's TOK), so nothing is gathered; larger calls copy their rows to slot order first,
+// and fp8 layers read the e4m3 planes that split_e4m3_kernel writes in slot order.
+bool tc_token_tiles(const TcLayer& L, int T) { return T <= kBNs[kNumBN - 1] && !L.w8; }
 
 // Calls whose groups fit one token tile read every weight byte once, so the weights go through L2
 // with an evict-first policy and leave it to what the next kernels of the call read again (rows,
@@ -1642,9 +1568,10 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
   a.a_rows_per_group = a.M;
   a.err = c.status;
   a.stream_a = streams_weights(c.T);
-  // the group layout is two or more launches old unless this kernel gathers the rows itself
-  // (then the permute is the previous launch)
-  a.prefetch_a = tc_gathers_in_kernel(L, c.T) && !shared ? 0 : 1;
+  // the group layout is two or more launches old unless nothing was copied in between (then the
+  // permute is the previous launch)
+  const bool tok = !shared && tc_token_tiles(L, c.T);
+  a.prefetch_a = tok ? 0 : 1;
   if (L.w8) {
     a.scale0 = shared ? L.ssg : L.sg;
     a.scale1 = shared ? L.ssu : L.su;
@@ -1652,8 +1579,8 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     a.b_lo_rows = shared ? L.Tmax : L.Tmax * L.K;
   }
   auto up_bn = [&](const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b, int grid) {
-    return L.w8 ? launch_up_bn<true>(bn, a0, a1, b, a, grid, st)
-                : launch_up_bn<false>(bn, a0, a1, b, a, grid, st);
+    return L.w8 ? launch_bn<kModeGateUp, true, false>(bn, a0, a1, b, a, grid, st)
+                : launch_bn<kModeGateUp, false, false>(bn, a0, a1, b, a, grid, st);
   };
   long long max_tiles;
   // the shared experts' unit set: every token of the call in order, weight 1 (reading R9)
@@ -1699,11 +1626,12 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
   max_tiles = (long long)(c.T * L.K + bn - 1) / bn + L.E;
   const long long units = max_tiles * a.m_tiles;
   const int grid = (int)std::min<long long>(L.num_sms, units);
-  if (tc_gathers_in_kernel(L, c.T)) {
-    // small call: the token rows are gathered from x inside the kernel
-    a.b_rows = c.perm_tok;
-    a.bx = (const __nv_bfloat16*)c.x;
-    return up_bn(m->wg, m->wu, m->wg, grid);
+  if (tok) {
+    a.slot_tok = c.perm_tok;
+    a.n_tok = c.T;
+    CUtensorMap xm;
+    if (!encode_2d(&xm, c.x, c.T, L.d, bn)) return cudaErrorInvalidValue;
+    return launch_bn<kModeGateUp, false, true>(bn, m->wg, m->wu, xm, a, grid, st);
   }
   if (pair && c.fold_shared && L.S > 0) {  // the shared experts in the same launch
     TcArgs sa;
@@ -1757,8 +1685,8 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
     a.b_lo_rows = shared ? L.S * L.Tmax : L.Tmax * L.K;
   }
   auto down_bn = [&](const CUtensorMap& a0, const CUtensorMap& b, int grid) {
-    return L.w8 ? launch_down_bn<true>(bn, a0, b, a, grid, st)
-                : launch_down_bn<false>(bn, a0, b, a, grid, st);
+    return L.w8 ? launch_bn<kModeDown, true, false>(bn, a0, a0, b, a, grid, st)
+                : launch_bn<kModeDown, false, false>(bn, a0, a0, b, a, grid, st);
   };
   long long max_tiles;
   auto shared_args = [&](TcArgs& s) {

@@ -59,7 +59,8 @@ int tc_bind(TcLayer& L, const eat_layer_desc& D, void* xperm, void* act, void* s
 void tc_destroy(TcLayer& L);
 int tc_tile_rows(const TcLayer& L, int T);       // gate/up token rows per tile, call of T tokens
 int tc_tile_rows_down(const TcLayer& L, int T);  // down-projection token rows per tile
-bool tc_gathers_in_kernel(const TcLayer& L, int T);  // gate/up gathers x rows itself (no Xperm)
+// The call's gate/up reads its token rows in token order (no row is copied to slot order).
+bool tc_token_tiles(const TcLayer& L, int T);
 // A call of T tokens runs its shared experts inside the routed SM-pair launches (TcCall's
 // fold_shared): one unit set after the other, one ramp and one tail per projection.
 bool tc_folds_shared(const TcLayer& L, int T);

@@ -379,6 +379,24 @@ def test_routing_and_account_outputs(which):
     B.close()
 
 
+def test_token_tiles_of_small_calls():
+    """bf16 gate/up tiles that hold the call's tokens in token order: token counts at and around the
+    tile widths, then a non-finite token among others (its column must not reach theirs)."""
+    lw = W.make_layer(OLMOE_S)
+    run_parity(OLMOE_S, lw, [1, 15, 16, 17, 33, 64, 65, 127, 128])
+    L = eat.EatLayer.from_workload(lw, 48, gpu_params(OLMOE_S))
+    x = W.make_tokens(OLMOE_S, 48).cuda()
+    want = L.forward(x, 0)
+    L.reset()
+    x[7, 3] = float("inf")
+    x[30, :] = float("nan")
+    got = L.forward(x, 0)
+    keep = [t for t in range(48) if t not in (7, 30)]
+    assert torch.equal(got[keep], want[keep])
+    assert torch.isnan(got[[7, 30]].float()).all()
+    L.close()
+
+
 @pytest.mark.parametrize("T", [127, 128, 129])
 def test_account_update_around_the_one_warp_limit(T):
     """Every token selects the same expert, so its account sums T slots: up to 128 by one warp,
