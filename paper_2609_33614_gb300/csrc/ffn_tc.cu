@@ -141,6 +141,14 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
+__device__ __forceinline__ void tma_load_4d_hint(void* dst, const CUtensorMap* map, uint64_t* bar,
+                                                 int c0, int c1, int c2, int c3, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2], %7;" ::"r"(smem_u32(dst)),
+      "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(policy)
+      : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
 }
@@ -227,16 +235,15 @@ __host__ __device__ constexpr int tmem_cols_for(int c) {
 
 // Kernel modes: the down projection (one A tile, plain epilogue); gate/up with two accumulators
 // (gate and up A tiles of 128 rows against one B tile, single-SM kernel); gate/up interleaved (one
-// A tile of 64 gate rows over the 64 up rows of the same features, one accumulator: an MMA covers
-// both projections of 64 features, and the epilogue pairs the gate and up warps of each feature;
-// SM-pair kernel).
+// A tile of 64 gate and 64 up rows of the same features, one accumulator: an MMA covers both
+// projections of 64 features, and the epilogue pairs the gate and up rows of each feature; SM-pair
+// kernel, and the single-SM kernel for token tiles of up to 64 rows).
 enum : int { kModeDown = 0, kModeGateUp = 1, kModeGateUpIL = 2 };
 
 template <int BN, int MODE, bool W8 = false>
 struct Cfg {
-  static_assert(MODE == kModeDown || MODE == kModeGateUp, "single-SM kernel modes");
-  static constexpr bool kGateUp = MODE == kModeGateUp;
-  static constexpr int kNA = kGateUp ? 2 : 1;
+  static constexpr bool kGateUp = MODE != kModeDown;
+  static constexpr int kNA = MODE == kModeGateUp ? 2 : 1;
   static constexpr int kNB = W8 ? 2 : 1;         // fp8: the B tile's e4m3 hi and lo parts
   static constexpr int kKB = W8 ? kBK8 : kBK;    // K elements of a k-block (128 B per row)
   static constexpr int kABytes = kBM * 128;
@@ -244,7 +251,10 @@ struct Cfg {
   static constexpr int kSubBytes = kNA * kABytes + kNB * kBBytes;  // one k-block's tiles
   // k-blocks per pipeline stage: a stage completes on one barrier phase, which costs ~0.6 µs
   // however few bytes it carries, so a stage carries two k-blocks wherever three such stages fit
-  static constexpr int kKPS = 6 * kSubBytes <= kSmemBudget - 2048 ? 2 : 1;
+  // (four where the 16-row interleaved gate/up tile leaves them that small)
+  static constexpr int kKPS = MODE == kModeGateUpIL && 12 * kSubBytes <= kSmemBudget - 2048 ? 4
+                              : 6 * kSubBytes <= kSmemBudget - 2048                          ? 2
+                                                                                             : 1;
   // e4m3 tiles of 64 or more tokens are drained by two warps per TMEM lane quarter (one per half
   // of the tile's columns), so an accumulator buffer returns to the MMA issuer sooner (e4m3
   // prefill +20 %)
@@ -390,7 +400,9 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
               const __grid_constant__ CUtensorMap mapB, const TcArgs args) {
   using C = Cfg<BN, MODE, W8>;
   constexpr bool GATEUP = C::kGateUp;
+  constexpr bool IL = MODE == kModeGateUpIL;  // A tile: 16-row interleave of 64 gate and 64 up rows
   constexpr int S = C::kStages;
+  static_assert(!IL || TOK, "the single-SM interleave is a layout of token tiles");
   static_assert(!TOK || (GATEUP && !W8), "token tiles are a layout of the bf16 gate/up");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -429,12 +441,14 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
   const uint64_t a_policy = policy_evict_first();
   // A tiles of one k-block: one 128-row box, or the gate and up boxes of the two accumulators
   auto load_a = [&](uint8_t* st, uint64_t* bar, int kb, int a_row) {
-    if (args.stream_a) {
+    if constexpr (IL) {
+      tma_load_4d_hint(st, &mapA0, bar, kb * C::kKB, 0, 0, a_row / 16, a_policy);
+    } else if (args.stream_a) {
       tma_load_2d_hint(st, &mapA0, bar, kb * C::kKB, a_row, a_policy);
-      if (GATEUP) tma_load_2d_hint(st + C::kABytes, &mapA1, bar, kb * C::kKB, a_row, a_policy);
+      if (C::kNA == 2) tma_load_2d_hint(st + C::kABytes, &mapA1, bar, kb * C::kKB, a_row, a_policy);
     } else {
       tma_load_2d(st, &mapA0, bar, kb * C::kKB, a_row);
-      if (GATEUP) tma_load_2d(st + C::kABytes, &mapA1, bar, kb * C::kKB, a_row);
+      if (C::kNA == 2) tma_load_2d(st + C::kABytes, &mapA1, bar, kb * C::kKB, a_row);
     }
   };
   __shared__ int32_t s_row[kMaxGroups + 1], s_tile[kMaxGroups + 1];
@@ -629,38 +643,63 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
       }
       const float* bsc = W8 ? args.bscale + (w.slot0 - w.g * args.b_shift_per_group) : nullptr;
       const int cend = min(cbeg + kCols, TOK ? args.n_tok : w.nrows);
-      for (int c0 = cbeg; c0 < cend; c0 += 16) {
-        if (TOK && !__any_sync(0xffffffffu, map[c0 - cbeg + (lane & 15)] >= 0)) continue;
-        uint32_t g[16], up[16];
-        tmem_ld16(tbase + c0, g);
-        if (GATEUP) tmem_ld16(tbase + C::kProjCols + c0, up);
-        if constexpr (C::kFuse) {  // + the lo parts' columns
-          uint32_t g2[16], up2[16];
-          tmem_ld16(tbase + BN + c0, g2);
-          if (GATEUP) tmem_ld16(tbase + C::kProjCols + BN + c0, up2);
+      if constexpr (IL) {
+        // lanes i and i + 16 hold the gate and up rows (in the order of the view) of feature
+        // 16 q + i; lanes 0-15 finish the first 8 columns of a chunk, lanes 16-31 the others, each
+        // with the other row's value from its partner
+        const bool lo = lane < 16, mine_is_gate = lo == (args.gate_first != 0);
+        const int fi = w.m0 + 16 * q + (lane & 15);
+        for (int c0 = cbeg; c0 < cend; c0 += 16) {
+          if (!__any_sync(0xffffffffu, map[c0 - cbeg + (lane & 15)] >= 0)) continue;
+          uint32_t v[16];
+          tmem_ld16(tbase + c0, v);
           tmem_wait_ld();
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            g[c] = __float_as_uint(__uint_as_float(g[c]) + __uint_as_float(g2[c]));
-            if (GATEUP) up[c] = __float_as_uint(__uint_as_float(up[c]) + __uint_as_float(up2[c]));
+          for (int j = 0; j < 8; ++j) {
+            const float mine = __uint_as_float(lo ? v[j] : v[j + 8]);
+            const float other =
+                __shfl_xor_sync(0xffffffffu, __uint_as_float(lo ? v[j + 8] : v[j]), 16);
+            const float gv = mine_is_gate ? mine : other, uv = mine_is_gate ? other : mine;
+            const int sl = map[c0 - cbeg + (lo ? j : j + 8)];
+            if (fi < args.M && sl >= 0)
+              ((__nv_bfloat16*)args.out)[(size_t)sl * args.M + fi] =
+                  __float2bfloat16_rn(silu_f(gv) * uv);
           }
         }
-        tmem_wait_ld();
-        if (fok) {
-#pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            const int sl = TOK ? map[c0 - cbeg + c] : w.slot0 + c0 + c;
-            if (TOK ? sl >= 0 : c0 + c < w.nrows) {
-              const size_t slot = (size_t)sl;
-              const float sc = W8 ? bsc[c0 + c] : 1.0f;
-              const float gv = W8 ? __uint_as_float(g[c]) * (s0 * sc) : __uint_as_float(g[c]);
-              if (GATEUP) {
-                const float uv = W8 ? __uint_as_float(up[c]) * (s1 * sc) : __uint_as_float(up[c]);
-                ((__nv_bfloat16*)args.out)[slot * args.M + f] = __float2bfloat16_rn(silu_f(gv) * uv);
-              } else if (args.out_bf16) {
-                ((__nv_bfloat16*)args.out)[slot * args.M + f] = __float2bfloat16_rn(gv);
-              } else {
-                ((float*)args.out)[(size_t)w.split * args.split_stride + slot * args.M + f] = gv;
+      } else {
+        for (int c0 = cbeg; c0 < cend; c0 += 16) {
+          if (TOK && !__any_sync(0xffffffffu, map[c0 - cbeg + (lane & 15)] >= 0)) continue;
+          uint32_t g[16], up[16];
+          tmem_ld16(tbase + c0, g);
+          if (GATEUP) tmem_ld16(tbase + C::kProjCols + c0, up);
+          if constexpr (C::kFuse) {  // + the lo parts' columns
+            uint32_t g2[16], up2[16];
+            tmem_ld16(tbase + BN + c0, g2);
+            if (GATEUP) tmem_ld16(tbase + C::kProjCols + BN + c0, up2);
+            tmem_wait_ld();
+  #pragma unroll
+            for (int c = 0; c < 16; ++c) {
+              g[c] = __float_as_uint(__uint_as_float(g[c]) + __uint_as_float(g2[c]));
+              if (GATEUP) up[c] = __float_as_uint(__uint_as_float(up[c]) + __uint_as_float(up2[c]));
+            }
+          }
+          tmem_wait_ld();
+          if (fok) {
+  #pragma unroll
+            for (int c = 0; c < 16; ++c) {
+              const int sl = TOK ? map[c0 - cbeg + c] : w.slot0 + c0 + c;
+              if (TOK ? sl >= 0 : c0 + c < w.nrows) {
+                const size_t slot = (size_t)sl;
+                const float sc = W8 ? bsc[c0 + c] : 1.0f;
+                const float gv = W8 ? __uint_as_float(g[c]) * (s0 * sc) : __uint_as_float(g[c]);
+                if (GATEUP) {
+                  const float uv = W8 ? __uint_as_float(up[c]) * (s1 * sc) : __uint_as_float(up[c]);
+                  ((__nv_bfloat16*)args.out)[slot * args.M + f] = __float2bfloat16_rn(silu_f(gv) * uv);
+                } else if (args.out_bf16) {
+                  ((__nv_bfloat16*)args.out)[slot * args.M + f] = __float2bfloat16_rn(gv);
+                } else {
+                  ((float*)args.out)[(size_t)w.split * args.split_stride + slot * args.M + f] = gv;
+                }
               }
             }
           }
@@ -1631,6 +1670,17 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     a.n_tok = c.T;
     CUtensorMap xm;
     if (!encode_2d(&xm, c.x, c.T, L.d, bn)) return cudaErrorInvalidValue;
+    // units of 64 features where the token tile is small beside the weights (it is read once more
+    // per feature): twice the units spread over the SMs more evenly.  us per call, 128 / 64
+    // features: OLMoE 1 token 38.6 / 37.0, 48 70.6 / 66.9, Mixtral 1 123.5 / 119.5, DeepSeek-V2-Lite
+    // 64 136.6 / 132.4; with 128-token tiles DeepSeek-V2-Lite 100 159.2 / 164.1, Qwen 100 80.6 / 83.9
+    if (m->il4 && bn <= 64) {
+      a.m_tile = kBM / 2;
+      a.m_tiles = (a.M + a.m_tile - 1) / a.m_tile;
+      a.gate_first = m->gate_first ? 1 : 0;
+      const int g2 = (int)std::min<long long>(L.num_sms, max_tiles * a.m_tiles);
+      return launch_bn<kModeGateUpIL, false, true>(bn, m->wgu4, m->wgu4, xm, a, g2, st);
+    }
     return launch_bn<kModeGateUp, false, true>(bn, m->wg, m->wu, xm, a, grid, st);
   }
   if (pair && c.fold_shared && L.S > 0) {  // the shared experts in the same launch
