@@ -732,8 +732,14 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
 constexpr int kPairBN = 256;
 constexpr int kPairRows = kPairBN / 2;
 
-template <int MODE, bool IL4 = false>
+// W8 (fp8 layers): the tile is 128 tokens; CTA 0 holds their hi rows of B and CTA 1 their lo rows, so
+// one MMA of N = 2 n multiplies the A tile with both (accumulator columns [0, n) and [n, 2 n), added
+// in the epilogue, n the unit's rows rounded up to 16) and each CTA stages 32 KB per 128-element
+// k-block where the single-SM kernel stages 48 (down) or 64 KB (gate/up) for the same MMAs.
+template <int MODE, bool IL4 = false, bool W8 = false>
 struct PairCfg {
+  static constexpr int kBN = W8 ? kPairRows : kPairBN;  // token rows of a unit
+  static constexpr int kKB = W8 ? kBK8 : kBK;           // K elements of a k-block
   static constexpr bool kIL = MODE == kModeGateUpIL;
   static constexpr int kABytes = kBM * kBK * 2;
   static constexpr int kBBytes = kPairRows * kBK * 2;
@@ -829,6 +835,20 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
 __host__ __device__ constexpr uint32_t idesc_bf16_pair(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
 }
+// The fp8 form: e4m3 operands, K = 32 per instruction (32 bytes of each row, as the bf16 form).
+__device__ __forceinline__ void mma_e4m3_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                              uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__host__ __device__ constexpr uint32_t idesc_e4m3_pair(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
+}
+// Token rows of an fp8 pair unit rounded up to 16: the lo parts' first accumulator column.
+__device__ __forceinline__ int pair_n8(int nrows) { return min(kPairRows, (nrows + 15) & ~15); }
 // MMA width of a pair unit: token rows rounded up to 32 (16 per CTA), at most 256.
 __device__ __forceinline__ int pair_n(int nrows) { return min(kPairBN, (nrows + 31) & ~31); }
 
@@ -840,15 +860,17 @@ __device__ __forceinline__ int pair_n(int nrows) { return min(kPairBN, (nrows + 
 // that alternates 16 gate rows and 16 up rows (mapA0; see encode_gu4), so each TMEM lane quarter
 // holds the gate and up rows of the same 16 features and the epilogue pairs them with shuffles
 // instead of the shared-memory exchange.
-template <int MODE, bool FOLD, bool IL4>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE, IL4>::kThreads, 1)
+template <int MODE, bool FOLD, bool IL4, bool W8>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE, IL4, W8>::kThreads, 1)
 tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                const __grid_constant__ CUtensorMap mapB, const TcArgs args,
                const __grid_constant__ CUtensorMap mapA0s, const __grid_constant__ CUtensorMap mapA1s,
                const __grid_constant__ CUtensorMap mapBs, const TcArgs args_s) {
-  using C = PairCfg<MODE, IL4>;
+  using C = PairCfg<MODE, IL4, W8>;
   constexpr bool IL = C::kIL;
+  constexpr int BN = C::kBN;
   static_assert(!IL4 || IL, "the 16-row interleave is a gate/up layout");
+  static_assert(!W8 || (IL4 == IL && !FOLD), "fp8: the 16-row interleave, one unit set");
   constexpr int S = C::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -898,7 +920,7 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int total_tiles = args.tile_offs
                               ? args.tile_offs[args.n_groups]
-                              : args.n_groups * ((args.uniform_rows + kPairBN - 1) / kPairBN);
+                              : args.n_groups * ((args.uniform_rows + BN - 1) / BN);
   const int units_r = total_tiles * args.m_tiles * args.n_split;
   const int units = units_r + (FOLD ? args_s.n_groups *
                                             ((args_s.uniform_rows + kPairBN - 1) / kPairBN) *
@@ -907,7 +929,7 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
   // unit u of the launch: the routed set first, then the shared one (true)
   auto unit_at = [&](int u, Unit& w) -> bool {
     if (!FOLD || u < units_r) {
-      w = decode_unit<kPairBN>(args, u, Offs{args.row_offs, args.tile_offs});
+      w = decode_unit<BN>(args, u, Offs{args.row_offs, args.tile_offs});
       return false;
     }
     w = decode_unit<kPairBN>(args_s, u - units_r, Offs{nullptr, nullptr});
@@ -933,7 +955,8 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         const int a_rows = sh ? args_s.a_rows_per_group : args.a_rows_per_group;
         const int b_shift = sh ? args_s.b_shift_per_group : args.b_shift_per_group;
         const int a_row = w.g * a_rows + w.m0 + (int)rank * C::kFeat;
-        const int b_row = w.slot0 - w.g * b_shift + (int)rank * (n / 2);
+        // (fp8: this CTA's plane of the tokens' rows)
+        const int b_row = w.slot0 - w.g * b_shift + (int)rank * (W8 ? args.b_lo_rows : n / 2);
         for (int kb = w.kb0; kb < w.kb1; kb += C::kKPS) {
           const int nk = min(C::kKPS, w.kb1 - kb);  // k-blocks of this stage
           if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, args.err, 1u, true)) {
@@ -947,7 +970,7 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           for (int j = 0; j < C::kKPS; ++j) {
             if (j < nk) {
               uint8_t* sj = st + j * C::kSubBytes;
-              const int kx = (kb + j) * kBK;
+              const int kx = (kb + j) * C::kKB;
               if (IL4) {
                 tma_load_4d_pair(sj, mA0, fb, kx, 0, 0, a_row / 16);
               } else if (IL) {
@@ -991,7 +1014,8 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         }
         tc_fence_after();
         const uint32_t d0 = tmem_base + (uint32_t)(buf * C::kAccCols);
-        const uint32_t idesc = idesc_bf16_pair(pair_n(w.nrows));
+        const uint32_t idesc = W8 ? idesc_e4m3_pair(2 * pair_n8(w.nrows))
+                                  : idesc_bf16_pair(pair_n(w.nrows));
         for (int kb = w.kb0; kb < w.kb1; kb += C::kKPS) {
           const int nk = min(C::kKPS, w.kb1 - kb);
           if (!mbar_wait(&full[stage], phase, abort_flag, args.err, 8u, true)) {
@@ -1005,9 +1029,11 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
               const uint32_t sa = smem_u32(smem + stage * C::kStageBytes + j * C::kSubBytes);
               const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sa + C::kABytes);
 #pragma unroll
-              for (int k = 0; k < kBK / 16; ++k)
-                mma_bf16_pair(d0, sdesc_step(da, k), sdesc_step(db, k), idesc,
-                              (kb > w.kb0 || j > 0 || k > 0) ? 1u : 0u);
+              for (int k = 0; k < 4; ++k) {
+                const uint32_t acc = (kb > w.kb0 || j > 0 || k > 0) ? 1u : 0u;
+                if (W8) mma_e4m3_pair(d0, sdesc_step(da, k), sdesc_step(db, k), idesc, acc);
+                else mma_bf16_pair(d0, sdesc_step(da, k), sdesc_step(db, k), idesc, acc);
+              }
             }
           }
           mma_commit_pair(&empty[stage]);
@@ -1048,11 +1074,26 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * C::kAccCols);
       const int f = w.m0 + (int)rank * C::kFeat + 16 * q + (lane & 15);
       const bool fok = f < M;
-      const int c_end = min(128 * ch + 128, w.nrows);
-      for (int c0 = 128 * ch; c0 < c_end; c0 += 32) {
+      float rs = 1.0f;  // fp8: the scale of this lane's weight row
+      if (W8 && fok) rs = (mine_is_gate ? args.scale0 : args.scale1)[(size_t)w.g * M + f];
+      const float* bsc = W8 ? args.bscale + (w.slot0 - w.g * args.b_shift_per_group) : nullptr;
+      constexpr int kCols = BN / 2;  // token columns of one warp
+      const int c_end = min(kCols * ch + kCols, w.nrows);
+      for (int c0 = kCols * ch; c0 < c_end; c0 += 32) {
         uint32_t v0[16], v1[16];
         tmem_ld16(tbase + c0, v0);
         tmem_ld16(tbase + c0 + 16, v1);
+        if constexpr (W8) {  // + the lo parts' columns, times the weight row's scale
+          uint32_t l0[16], l1[16];
+          tmem_ld16(tbase + pair_n8(w.nrows) + c0, l0);
+          tmem_ld16(tbase + pair_n8(w.nrows) + c0 + 16, l1);
+          tmem_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            v0[j] = __float_as_uint((__uint_as_float(v0[j]) + __uint_as_float(l0[j])) * rs);
+            v1[j] = __float_as_uint((__uint_as_float(v1[j]) + __uint_as_float(l1[j])) * rs);
+          }
+        }
         tmem_wait_ld();
         const int cb = c0 + (lo ? 0 : 16);
 #pragma unroll
@@ -1060,10 +1101,16 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           const float mine = __uint_as_float(lo ? v0[j] : v1[j]);
           const float other =
               __shfl_xor_sync(0xffffffffu, __uint_as_float(lo ? v1[j] : v0[j]), 16);
-          const float g = mine_is_gate ? mine : other;
-          const float up = mine_is_gate ? other : mine;
-          if (fok && cb + j < w.nrows)
+          float g = mine_is_gate ? mine : other;
+          float up = mine_is_gate ? other : mine;
+          if (fok && cb + j < w.nrows) {
+            if (W8) {
+              const float sc = bsc[cb + j];
+              g *= sc;
+              up *= sc;
+            }
             out[(size_t)(w.slot0 + cb + j) * M + f] = __float2bfloat16_rn(silu_f(g) * up);
+          }
         }
       }
       tc_fence_before();
@@ -1164,10 +1211,24 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * C::kAccCols);
       const int f = w.m0 + (int)rank * C::kFeat + 32 * q + lane;
       const bool fok = f < M;
-      const int c_end = min(128 * ch + 128, w.nrows);
-      for (int c0 = 128 * ch; c0 < c_end; c0 += 16) {
+      float rs = 1.0f;  // fp8: the scale of this lane's weight row
+      if (W8 && fok) rs = args.scale0[(size_t)w.g * M + f];
+      const float* bsc = W8 ? args.bscale + (w.slot0 - w.g * args.b_shift_per_group) : nullptr;
+      constexpr int kCols = BN / 2;  // token columns of one warp
+      const int c_end = min(kCols * ch + kCols, w.nrows);
+      for (int c0 = kCols * ch; c0 < c_end; c0 += 16) {
         uint32_t g[16];
         tmem_ld16(tbase + c0, g);
+        if constexpr (W8) {  // + the lo parts' columns
+          uint32_t l[16];
+          tmem_ld16(tbase + pair_n8(w.nrows) + c0, l);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < 16; ++c)
+            if (c0 + c < w.nrows)
+              g[c] = __float_as_uint((__uint_as_float(g[c]) + __uint_as_float(l[c])) *
+                                     (rs * bsc[c0 + c]));
+        }
         tmem_wait_ld();
         if (fok) {
 #pragma unroll
@@ -1285,7 +1346,7 @@ bool encode_2d_u8(CUtensorMap* m, const void* ptr, long long rows, long long col
 // rows.  The two allocations need not be adjacent: the h stride is their distance.  false when
 // the view cannot be encoded (the caller then keeps the two 64-row boxes).
 bool encode_gu4(CUtensorMap* m, const void* gate, const void* up, long long rows, long long cols,
-                bool* gate_first) {
+                bool* gate_first, bool e4m3 = false) {
   auto fn = encode_fn();
   if (!fn || rows % 16 != 0 || gate == up) return false;
   const bool gf = (uintptr_t)gate < (uintptr_t)up;
@@ -1294,11 +1355,12 @@ bool encode_gu4(CUtensorMap* m, const void* gate, const void* up, long long rows
   const unsigned long long dist = (unsigned long long)(hi - lo);
   if (dist % 16 != 0 || dist >= (1ULL << 40)) return false;
   cuuint64_t dims[4] = {(cuuint64_t)cols, 16, 2, (cuuint64_t)(rows / 16)};
-  cuuint64_t strides[3] = {(cuuint64_t)cols * 2, (cuuint64_t)dist, (cuuint64_t)cols * 2 * 16};
-  cuuint32_t box[4] = {(cuuint32_t)kBK, 16, 2, 4};
+  const cuuint64_t pitch = (cuuint64_t)cols * (e4m3 ? 1 : 2);
+  cuuint64_t strides[3] = {pitch, (cuuint64_t)dist, pitch * 16};
+  cuuint32_t box[4] = {(cuuint32_t)(e4m3 ? kBK8 : kBK), 16, 2, 4};  // 128 bytes of each row
   cuuint32_t estr[4] = {1, 1, 1, 1};
-  const bool ok = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<char*>(lo), dims, strides,
-                     box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  const bool ok = fn(m, e4m3 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
+                     const_cast<char*>(lo), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   *gate_first = gf;
@@ -1343,17 +1405,17 @@ cudaError_t launch_tc(const CUtensorMap& a0, const CUtensorMap& a1, const CUtens
 // SM-pair kernels: one 2-CTA cluster per pair of SMs, at most as many pairs as can be resident.
 // The routed set (a0, a1, b, args) and, when sargs is given, the shared set of the same call in
 // the same launch; units counts both.
-template <int MODE, bool FOLD, bool IL4>
+template <int MODE, bool FOLD, bool IL4, bool W8 = false>
 cudaError_t launch_pair_t(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
                           const TcArgs& args, long long units, int num_sms, cudaStream_t st,
                           const CUtensorMap* sa0, const CUtensorMap* sa1, const CUtensorMap* sb,
                           const TcArgs* sargs) {
-  using C = PairCfg<MODE, IL4>;
+  using C = PairCfg<MODE, IL4, W8>;
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   static int max_pairs = 0;
   std::call_once(once, [num_sms] {
-    attr_err = cudaFuncSetAttribute(tc_pair_kernel<MODE, FOLD, IL4>,
+    attr_err = cudaFuncSetAttribute(tc_pair_kernel<MODE, FOLD, IL4, W8>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
     if (attr_err != cudaSuccess) return;
     cudaLaunchConfig_t cfg = {};
@@ -1368,7 +1430,7 @@ cudaError_t launch_pair_t(const CUtensorMap& a0, const CUtensorMap& a1, const CU
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<MODE, FOLD, IL4>, &cfg) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<MODE, FOLD, IL4, W8>, &cfg) != cudaSuccess ||
         n <= 0) {
       cudaGetLastError();
       n = num_sms / 2;
@@ -1380,7 +1442,7 @@ cudaError_t launch_pair_t(const CUtensorMap& a0, const CUtensorMap& a1, const CU
   if (pairs <= 0) return cudaSuccess;
   TcArgs none;
   std::memset(&none, 0, sizeof(none));
-  return launch_pdl(tc_pair_kernel<MODE, FOLD, IL4>, dim3((unsigned)(2 * pairs)), dim3(C::kThreads),
+  return launch_pdl(tc_pair_kernel<MODE, FOLD, IL4, W8>, dim3((unsigned)(2 * pairs)), dim3(C::kThreads),
                     C::kSmemBytes, st, a0, a1, b, args, sa0 ? *sa0 : a0, sa1 ? *sa1 : a1,
                     sb ? *sb : b, sargs ? *sargs : none);
 }
@@ -1394,6 +1456,14 @@ cudaError_t launch_pair(const CUtensorMap& a0, const CUtensorMap& a1, const CUte
                                           sargs);
   return launch_pair_t<MODE, false, IL4>(a0, a1, b, args, units, num_sms, st, nullptr, nullptr,
                                          nullptr, nullptr);
+}
+
+// fp8: one unit set (the gate/up map is the 16-row interleaved view).
+template <int MODE>
+cudaError_t launch_pair8(const CUtensorMap& a, const CUtensorMap& b, const TcArgs& args,
+                         long long units, int num_sms, cudaStream_t st) {
+  return launch_pair_t<MODE, false, MODE == kModeGateUpIL, true>(a, a, b, args, units, num_sms, st,
+                                                                 nullptr, nullptr, nullptr, nullptr);
 }
 
 // Single-SM launches: token tiles of 16..128 rows (256-row tiles run on SM pairs); W8 for fp8
@@ -1440,6 +1510,11 @@ bool tc_token_tiles(const TcLayer& L, int T) { return T <= kBNs[kNumBN - 1] && !
 // group's later tiles find its weights in L2: Qwen 333 tokens 140.8 / 141.2, e4m3 OLMoE 3001 tokens
 // 386.6 / 390.1.
 static int streams_weights(int T) { return T <= kBNs[kNumBN - 1] ? 1 : 0; }
+
+// fp8 calls on SM pairs (128-token tiles): every call whose tokens do not fit one tile.  us per
+// call, single SM / pairs: OLMoE 200 tokens 90.7 / 87.1, 3001 379.5 / 364.6, Mixtral shape 400 385.3
+// / 358.6, 1000 660.7 / 620.7, Qwen 333 105.9 / 101.9, DeepSeek-V2-Lite 600 170.0 / 169.8.
+static bool pairs8(const TcLayer& L, int T) { return L.w8 && T > kBNs[kNumBN - 1]; }
 
 bool tc_folds_shared(const TcLayer& L, int T) {
   return L.S > 0 && !L.w8 && tc_tile_rows(L, T) == kPairBN;
@@ -1535,6 +1610,12 @@ int tc_bind(TcLayer& L, const eat_layer_desc& D, void* xperm, void* act, void* s
       ok = encode_2d_u8(&m->wsg, D.ws_gate, (long long)L.S * L.Fs, L.d, kBM) &&
            encode_2d_u8(&m->wsu, D.ws_up, (long long)L.S * L.Fs, L.d, kBM) &&
            encode_2d_u8(&m->wsd, D.ws_down, (long long)L.S * L.d, L.Fs, kBM);
+    if (ok)
+      m->il4 = encode_gu4(&m->wgu4, D.w_gate, D.w_up, (long long)L.E * L.F, L.d, &m->gate_first,
+                          true);
+    if (ok && L.S > 0)
+      m->sil4 = encode_gu4(&m->wsgu4, D.ws_gate, D.ws_up, (long long)L.S * L.Fs, L.d,
+                           &m->sgate_first, true);
   } else {
     ok = encode_2d(&m->wg, D.w_gate, (long long)L.E * L.F, L.d, kBM) &&
          encode_2d(&m->wu, D.w_up, (long long)L.E * L.F, L.d, kBM) &&
@@ -1642,6 +1723,23 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     s.b_shift_per_group = c.T;
     s.out = c.sact;
   };
+  if (L.w8 && pairs8(L, c.T) && (shared ? m->sil4 : m->il4)) {
+    if (shared) {
+      shared_args(a);
+      a.gate_first = m->sgate_first ? 1 : 0;
+      return launch_pair8<kModeGateUpIL>(m->wsgu4, m->xqt[bn_index(kPairRows)], a,
+                                         (long long)L.S * ((c.T + bn - 1) / bn) * a.m_tiles,
+                                         L.num_sms, st);
+    }
+    a.gate_first = m->gate_first ? 1 : 0;
+    a.n_groups = L.E;
+    a.row_offs = c.offs;
+    a.tile_offs = c.tile_offs;
+    a.out = c.act;
+    return launch_pair8<kModeGateUpIL>(m->wgu4, m->xq[bn_index(kPairRows)], a,
+                                       ((long long)(c.T * L.K + bn - 1) / bn + L.E) * a.m_tiles,
+                                       L.num_sms, st);
+  }
   if (shared) {
     CUtensorMap xm;
     if (L.w8) xm = m->xqt[bn_index(bn)];
@@ -1717,7 +1815,8 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
   TcArgs a;
   std::memset(&a, 0, sizeof(a));
   const int bn = c.tile_rows_down;
-  const bool pair = bn == kPairBN;  // SM pairs: 256 output features per unit
+  const bool pair8 = L.w8 && pairs8(L, c.T);
+  const bool pair = bn == kPairBN || pair8;  // SM pairs: 256 output features per unit
   const int Kdim = shared ? L.Fs : L.F;
   a.M = L.d;
   a.m_tile = pair ? 2 * kBM : kBM;
@@ -1763,6 +1862,8 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
     a.kb_per_split = (a.kblocks + n_split - 1) / n_split;
     max_tiles = (long long)L.S * ((c.T + bn - 1) / bn);
     const long long units = max_tiles * a.m_tiles;
+    if (pair8)
+      return launch_pair8<kModeDown>(m->wsd, m->saq[bn_index(kPairRows)], a, units, L.num_sms, st);
     if (pair)
       return launch_pair<kModeDown>(m->wsd, m->wsd, m->sact[bn_index(kPairRows)], a, units,
                                     L.num_sms, st);
@@ -1785,6 +1886,8 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
                                   L.num_sms, st, &m->wsd, &m->wsd,
                                   &m->sact[bn_index(kPairRows)], &sa);
   }
+  if (pair8)
+    return launch_pair8<kModeDown>(m->wd, m->aq[bn_index(kPairRows)], a, units, L.num_sms, st);
   if (pair)
     return launch_pair<kModeDown>(m->wd, m->wd, m->act[bn_index(kPairRows)], a, units, L.num_sms,
                                   st);

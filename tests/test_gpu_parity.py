@@ -446,6 +446,21 @@ def test_fp8_large_calls_small_groups(E, K, T):
     layer.close()
 
 
+@pytest.mark.parametrize("d,F,E,K,S,Ts", [
+    (192, 320, 6, 2, 2, [129, 300]),    # ragged last k-blocks, partial feature tiles, shared experts
+    (256, 1024, 64, 4, 0, [130, 700]),  # mostly partial tiles, down projections split along K
+])
+def test_fp8_sm_pairs(d, F, E, K, S, Ts):
+    """e4m3 layers on SM pairs (calls above 128 tokens): the hi rows in one CTA, the lo rows in the
+    other, 128-token tiles of every width."""
+    sh = W.scaled(W.QWEN if S else W.OLMOE, f"p8-{d}", d_model=d, n_experts=E, d_ff=F, max_k=K,
+                  n_shared=S, d_ff_shared=F if S else 0)
+    lw8 = W.to_fp8(W.make_layer(sh))
+    layer = eat.EatLayer.from_workload(lw8, max(Ts), gpu_params(sh))
+    run_parity(sh, lw8.dequantized(), Ts, layer=layer)
+    layer.close()
+
+
 def test_fp8_large_call_one_group():
     """e4m3 weights, one expert takes all 2100 tokens: 16 full 128-token tiles and a partial one."""
     lw = W.make_layer(OLMOE_S)
