@@ -110,8 +110,13 @@ def _ptr(t):
 
 
 def _stream(stream):
+    """The stream's handle; None: torch's current stream.  The raw query saves most of what building
+    a Stream object costs the host on each call (a small call is bound by the host)."""
     if stream is None:
         import torch
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is not None:
+            return raw(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream
 
