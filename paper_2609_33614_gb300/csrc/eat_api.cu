@@ -508,9 +508,12 @@ eat_status eat_create(const eat_layer_desc* desc, const eat_params* params, eat_
     h->opart_rows = tc_opart_rows(h->tc);
   }
 
+  // (the split depends on the call's number of 64-token tiles, so the largest T of each counts)
   int max_lsplit = 0;
-  for (int T = 1; T <= h->Tmax; ++T)
+  for (int T0 = 0; T0 < h->Tmax; T0 += kRouterTileT) {
+    const int T = std::min(h->Tmax, T0 + kRouterTileT);
     max_lsplit = std::max(max_lsplit, router_split(T, h->d, h->E) * T);
+  }
 
   const size_t rows = (size_t)h->Tmax * h->K;
   struct Part { void** p; size_t bytes; };

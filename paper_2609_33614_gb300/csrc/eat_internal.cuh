@@ -135,6 +135,7 @@ cudaError_t launch_route_select(const float2* part, int n_split, const float* b_
                                 int E, int K, const int64_t* accN, const double* accP,
                                 const double* accC, RouteParams rp, int32_t* idx, float* w,
                                 int32_t* k, float* psel, cudaStream_t st);
+constexpr int kRouterTileT = 64;    // tokens of a tile of the larger calls' routers
 constexpr int kSmallRouterT = 128;  // calls up to this many tokens use the GEMV-style router
 int router_split(int T, int d, int E);
 

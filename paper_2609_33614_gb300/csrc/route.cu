@@ -39,7 +39,7 @@ __device__ __forceinline__ float load_x(const __nv_bfloat16* p, size_t i) {
 // with 4 tokens x 4 experts each.  x and W_r chunks of 32 columns are staged transposed in shared
 // memory; every output takes 32 fp32 FMAs per chunk and the chunk sums are added with Kahan
 // compensation (fp32), so the score carries about the error of an fp64 sum of fp32 products.
-constexpr int kTileT = 64, kTileE = 64, kChunkK = 32;
+constexpr int kTileT = kRouterTileT, kTileE = 64, kChunkK = 32;
 
 __device__ __forceinline__ void kahan_add(float& sum, float& comp, float v) {
   const float y = v - comp;
@@ -202,7 +202,7 @@ router_logits_small_kernel(const TX* __restrict__ x, const float* __restrict__ w
 // fixed number of slices for every tile.  x and W_r go through a three-stage shared-memory ring
 // as fp32 (row stride 36 floats): W_r by cp.async, x through registers (converted when stored),
 // two units ahead; one block barrier per unit.
-constexpr int kSKT = 64, kSKE = 64, kSKS = kChunkK + 4, kSKStages = 3;
+constexpr int kSKT = kRouterTileT, kSKE = 64, kSKS = kChunkK + 4, kSKStages = 3;
 constexpr int kSKTM = 4;        // tokens per thread: 256 threads, two CTAs per SM
 // Columns of d per CTA at least: 256, or 128 while the grid is no larger than the SM count (more CTAs
 // cut the run of a call that does not fill the GPU; beyond that the selection loses more to the
@@ -1034,6 +1034,9 @@ bool sk_eligible(int T, int d) { return T > kSmallT && d % kChunkK == 0; }
 
 }  // namespace
 
+// (eat_create relies on the split of a call being the same for all T with the same number of
+// kRouterTileT-token tiles, up to kSmallRouterT and beyond it)
+static_assert(kSmallT % kRouterTileT == 0, "the small calls end at a tile");
 int router_split(int T, int d, int E) {
   if (T <= kSmallT) return (d + kSmallSlice - 1) / kSmallSlice;
   if (sk_eligible(T, d)) {
