@@ -736,17 +736,17 @@ constexpr int kPairRows = kPairBN / 2;
 // one MMA of N = 2 n multiplies the A tile with both (accumulator columns [0, n) and [n, 2 n), added
 // in the epilogue, n the unit's rows rounded up to 16) and each CTA stages 32 KB per 128-element
 // k-block where the single-SM kernel stages 48 (down) or 64 KB (gate/up) for the same MMAs.
-template <int MODE, bool IL4 = false, bool W8 = false>
+template <int MODE, bool IL4 = false, bool W8 = false, int KPS = 2>
 struct PairCfg {
   static constexpr int kBN = W8 ? kPairRows : kPairBN;  // token rows of a unit
   static constexpr int kKB = W8 ? kBK8 : kBK;           // K elements of a k-block
   static constexpr bool kIL = MODE == kModeGateUpIL;
   static constexpr int kABytes = kBM * kBK * 2;
   static constexpr int kBBytes = kPairRows * kBK * 2;
-  // k-blocks per pipeline stage: each stage completes on one barrier phase, and a phase costs
-  // ~0.6 µs however few bytes it carries, so a stage carries two k-blocks' A and B tiles (64 KB
-  // per CTA)
-  static constexpr int kKPS = 2;
+  // k-blocks per pipeline stage: two (three stages of 64 KB), or one (seven of 32 KB: a stage comes
+  // back sooner and more are in flight, but the MMA thread waits and commits twice as often).  One
+  // pays where tiles are mostly partial and the stages' round trip is the pace (see pair_one_kb).
+  static constexpr int kKPS = KPS;
   static constexpr int kSubBytes = kABytes + kBBytes;  // one k-block's A and B tiles
   static constexpr int kStageBytes = kKPS * kSubBytes;
   // TMEM is drained by two warps per lane quarter, one per half of the 256 token columns: the
@@ -860,13 +860,14 @@ __device__ __forceinline__ int pair_n(int nrows) { return min(kPairBN, (nrows + 
 // that alternates 16 gate rows and 16 up rows (mapA0; see encode_gu4), so each TMEM lane quarter
 // holds the gate and up rows of the same 16 features and the epilogue pairs them with shuffles
 // instead of the shared-memory exchange.
-template <int MODE, bool FOLD, bool IL4, bool W8>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PairCfg<MODE, IL4, W8>::kThreads, 1)
+template <int MODE, bool FOLD, bool IL4, bool W8, int KPS>
+__global__ void __cluster_dims__(2, 1, 1)
+__launch_bounds__(PairCfg<MODE, IL4, W8, KPS>::kThreads, 1)
 tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                const __grid_constant__ CUtensorMap mapB, const TcArgs args,
                const __grid_constant__ CUtensorMap mapA0s, const __grid_constant__ CUtensorMap mapA1s,
                const __grid_constant__ CUtensorMap mapBs, const TcArgs args_s) {
-  using C = PairCfg<MODE, IL4, W8>;
+  using C = PairCfg<MODE, IL4, W8, KPS>;
   constexpr bool IL = C::kIL;
   constexpr int BN = C::kBN;
   static_assert(!IL4 || IL, "the 16-row interleave is a gate/up layout");
@@ -1405,17 +1406,17 @@ cudaError_t launch_tc(const CUtensorMap& a0, const CUtensorMap& a1, const CUtens
 // SM-pair kernels: one 2-CTA cluster per pair of SMs, at most as many pairs as can be resident.
 // The routed set (a0, a1, b, args) and, when sargs is given, the shared set of the same call in
 // the same launch; units counts both.
-template <int MODE, bool FOLD, bool IL4, bool W8 = false>
+template <int MODE, bool FOLD, bool IL4, bool W8 = false, int KPS = 2>
 cudaError_t launch_pair_t(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
                           const TcArgs& args, long long units, int num_sms, cudaStream_t st,
                           const CUtensorMap* sa0, const CUtensorMap* sa1, const CUtensorMap* sb,
                           const TcArgs* sargs) {
-  using C = PairCfg<MODE, IL4, W8>;
+  using C = PairCfg<MODE, IL4, W8, KPS>;
   static std::once_flag once;
   static cudaError_t attr_err = cudaSuccess;
   static int max_pairs = 0;
   std::call_once(once, [num_sms] {
-    attr_err = cudaFuncSetAttribute(tc_pair_kernel<MODE, FOLD, IL4, W8>,
+    attr_err = cudaFuncSetAttribute(tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
     if (attr_err != cudaSuccess) return;
     cudaLaunchConfig_t cfg = {};
@@ -1430,7 +1431,7 @@ cudaError_t launch_pair_t(const CUtensorMap& a0, const CUtensorMap& a1, const CU
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<MODE, FOLD, IL4, W8>, &cfg) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>, &cfg) != cudaSuccess ||
         n <= 0) {
       cudaGetLastError();
       n = num_sms / 2;
@@ -1442,20 +1443,34 @@ cudaError_t launch_pair_t(const CUtensorMap& a0, const CUtensorMap& a1, const CU
   if (pairs <= 0) return cudaSuccess;
   TcArgs none;
   std::memset(&none, 0, sizeof(none));
-  return launch_pdl(tc_pair_kernel<MODE, FOLD, IL4, W8>, dim3((unsigned)(2 * pairs)), dim3(C::kThreads),
+  return launch_pdl(tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>, dim3((unsigned)(2 * pairs)), dim3(C::kThreads),
                     C::kSmemBytes, st, a0, a1, b, args, sa0 ? *sa0 : a0, sa1 ? *sa1 : a1,
                     sb ? *sb : b, sargs ? *sargs : none);
 }
-template <int MODE, bool IL4 = false>
-cudaError_t launch_pair(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
-                        const TcArgs& args, long long units, int num_sms, cudaStream_t st,
-                        const CUtensorMap* sa0 = nullptr, const CUtensorMap* sa1 = nullptr,
-                        const CUtensorMap* sb = nullptr, const TcArgs* sargs = nullptr) {
+// KPS: k-blocks per pipeline stage (one only for the 16-row interleaved gate/up and the down
+// projection, whose shared memory holds seven stages).
+template <int MODE, bool IL4, int KPS>
+cudaError_t launch_pair_k(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
+                          const TcArgs& args, long long units, int num_sms, cudaStream_t st,
+                          const CUtensorMap* sa0, const CUtensorMap* sa1, const CUtensorMap* sb,
+                          const TcArgs* sargs) {
   if (sargs)
-    return launch_pair_t<MODE, true, IL4>(a0, a1, b, args, units, num_sms, st, sa0, sa1, sb,
-                                          sargs);
-  return launch_pair_t<MODE, false, IL4>(a0, a1, b, args, units, num_sms, st, nullptr, nullptr,
-                                         nullptr, nullptr);
+    return launch_pair_t<MODE, true, IL4, false, KPS>(a0, a1, b, args, units, num_sms, st, sa0, sa1,
+                                                      sb, sargs);
+  return launch_pair_t<MODE, false, IL4, false, KPS>(a0, a1, b, args, units, num_sms, st, nullptr,
+                                                     nullptr, nullptr, nullptr);
+}
+template <int MODE, bool IL4 = false>
+cudaError_t launch_pair(bool one_kb, const CUtensorMap& a0, const CUtensorMap& a1,
+                        const CUtensorMap& b, const TcArgs& args, long long units, int num_sms,
+                        cudaStream_t st, const CUtensorMap* sa0 = nullptr,
+                        const CUtensorMap* sa1 = nullptr, const CUtensorMap* sb = nullptr,
+                        const TcArgs* sargs = nullptr) {
+  if constexpr (IL4 || MODE == kModeDown) {
+    if (one_kb)
+      return launch_pair_k<MODE, IL4, 1>(a0, a1, b, args, units, num_sms, st, sa0, sa1, sb, sargs);
+  }
+  return launch_pair_k<MODE, IL4, 2>(a0, a1, b, args, units, num_sms, st, sa0, sa1, sb, sargs);
 }
 
 // fp8: one unit set (the gate/up map is the 16-row interleaved view).
@@ -1515,6 +1530,15 @@ static int streams_weights(int T) { return T <= kBNs[kNumBN - 1] ? 1 : 0; }
 // call, single SM / pairs: OLMoE 200 tokens 90.7 / 87.1, 3001 379.5 / 364.6, Mixtral shape 400 385.3
 // / 358.6, 1000 660.7 / 620.7, Qwen 333 105.9 / 101.9, DeepSeek-V2-Lite 600 170.0 / 169.8.
 static bool pairs8(const TcLayer& L, int T) { return L.w8 && T > kBNs[kNumBN - 1]; }
+
+// bf16 SM pairs: one k-block per stage for calls of at most 512 rows per expert on average.  us per
+// call, two / one: OLMoE 600 tokens 158.8 / 154.6, 4096 (512 rows) 410.8 / 403.8, 10000 (1250) 861 /
+// 868; Mixtral shape 400 534 / 514, 2000 (500) 1236 / 1183; DeepSeek-V2-Lite 1500 309 / 296, 4096
+// (384) 516 / 511, 16384 (1536) 1685 / 1692; Qwen 1000 202 / 197, 8192 (546, beside shared experts'
+// full tiles) 844 / 871.
+static bool pair_one_kb(const TcLayer& L, int T) {
+  return (long long)T * L.K <= 512LL * L.E;
+}
 
 bool tc_folds_shared(const TcLayer& L, int T) {
   return L.S > 0 && !L.w8 && tc_tile_rows(L, T) == kPairBN;
@@ -1679,6 +1703,7 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
   std::memset(&a, 0, sizeof(a));
   const int bn = c.tile_rows;
   const bool pair = bn == kPairBN;  // SM pairs, interleaved gate/up: 128 features per unit
+  const bool one_kb = pair_one_kb(L, c.T);
   a.M = shared ? L.Fs : L.F;
   a.m_tile = kBM;
   a.m_tiles = (a.M + a.m_tile - 1) / a.m_tile;
@@ -1749,10 +1774,11 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     const long long units = max_tiles * a.m_tiles;
     if (pair && m->sil4) {
       a.gate_first = m->sgate_first ? 1 : 0;
-      return launch_pair<kModeGateUpIL, true>(m->wsgu4, m->wsgu4, xm, a, units, L.num_sms, st);
+      return launch_pair<kModeGateUpIL, true>(one_kb, m->wsgu4, m->wsgu4, xm, a, units, L.num_sms,
+                                              st);
     }
     if (pair)
-      return launch_pair<kModeGateUpIL>(m->wsg64, m->wsu64, xm, a, units, L.num_sms, st);
+      return launch_pair<kModeGateUpIL>(one_kb, m->wsg64, m->wsu64, xm, a, units, L.num_sms, st);
     const int grid = (int)std::min<long long>(L.num_sms, units);
     return up_bn(m->wsg, m->wsu, xm, grid);
   }
@@ -1790,22 +1816,22 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     if (m->il4 && m->sil4) {
       a.gate_first = m->gate_first ? 1 : 0;
       sa.gate_first = m->sgate_first ? 1 : 0;
-      return launch_pair<kModeGateUpIL, true>(m->wgu4, m->wgu4, m->xperm[bn_index(kPairRows)], a,
-                                              units + s_units, L.num_sms, st, &m->wsgu4,
-                                              &m->wsgu4, &xm, &sa);
+      return launch_pair<kModeGateUpIL, true>(one_kb, m->wgu4, m->wgu4,
+                                              m->xperm[bn_index(kPairRows)], a, units + s_units,
+                                              L.num_sms, st, &m->wsgu4, &m->wsgu4, &xm, &sa);
     }
-    return launch_pair<kModeGateUpIL>(m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
+    return launch_pair<kModeGateUpIL>(one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
                                       units + s_units, L.num_sms, st, &m->wsg64, &m->wsu64, &xm,
                                       &sa);
   }
   if (pair && m->il4) {
     a.gate_first = m->gate_first ? 1 : 0;
-    return launch_pair<kModeGateUpIL, true>(m->wgu4, m->wgu4, m->xperm[bn_index(kPairRows)], a,
-                                            units, L.num_sms, st);
+    return launch_pair<kModeGateUpIL, true>(one_kb, m->wgu4, m->wgu4,
+                                            m->xperm[bn_index(kPairRows)], a, units, L.num_sms, st);
   }
   if (pair)
-    return launch_pair<kModeGateUpIL>(m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a, units,
-                                      L.num_sms, st);
+    return launch_pair<kModeGateUpIL>(one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
+                                      units, L.num_sms, st);
   return up_bn(m->wg, m->wu, L.w8 ? m->xq[bn_index(bn)] : m->xperm[bn_index(bn)], grid);
 }
 
@@ -1817,6 +1843,7 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
   const int bn = c.tile_rows_down;
   const bool pair8 = L.w8 && pairs8(L, c.T);
   const bool pair = bn == kPairBN || pair8;  // SM pairs: 256 output features per unit
+  const bool one_kb = pair_one_kb(L, c.T);
   const int Kdim = shared ? L.Fs : L.F;
   a.M = L.d;
   a.m_tile = pair ? 2 * kBM : kBM;
@@ -1865,7 +1892,7 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
     if (pair8)
       return launch_pair8<kModeDown>(m->wsd, m->saq[bn_index(kPairRows)], a, units, L.num_sms, st);
     if (pair)
-      return launch_pair<kModeDown>(m->wsd, m->wsd, m->sact[bn_index(kPairRows)], a, units,
+      return launch_pair<kModeDown>(one_kb, m->wsd, m->wsd, m->sact[bn_index(kPairRows)], a, units,
                                     L.num_sms, st);
     const int grid = (int)std::min<long long>(L.num_sms, units);
     return down_bn(m->wsd, L.w8 ? m->saq[bn_index(bn)] : m->sact[bn_index(bn)], grid);
@@ -1882,14 +1909,16 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
     TcArgs sa;
     shared_args(sa);
     const long long s_units = (long long)L.S * ((c.T + bn - 1) / bn) * sa.m_tiles;
-    return launch_pair<kModeDown>(m->wd, m->wd, m->act[bn_index(kPairRows)], a, units + s_units,
+    return launch_pair<kModeDown>(one_kb, m->wd, m->wd, m->act[bn_index(kPairRows)], a,
+                                  units + s_units,
                                   L.num_sms, st, &m->wsd, &m->wsd,
                                   &m->sact[bn_index(kPairRows)], &sa);
   }
   if (pair8)
     return launch_pair8<kModeDown>(m->wd, m->aq[bn_index(kPairRows)], a, units, L.num_sms, st);
   if (pair)
-    return launch_pair<kModeDown>(m->wd, m->wd, m->act[bn_index(kPairRows)], a, units, L.num_sms,
+    return launch_pair<kModeDown>(one_kb, m->wd, m->wd, m->act[bn_index(kPairRows)], a, units,
+                                  L.num_sms,
                                   st);
   const int grid = (int)std::min<long long>(L.num_sms, units);
   return down_bn(m->wd, L.w8 ? m->aq[bn_index(bn)] : m->act[bn_index(bn)], grid);

@@ -427,6 +427,15 @@ def test_sm_pair_smallest_calls(E, K, S, T):
     run_parity(sh, W.make_layer(sh), [T, T - 1])
 
 
+@pytest.mark.parametrize("T", [1000, 1100])
+def test_sm_pair_stage_sizes(T):
+    """Calls of at most 512 rows per expert run one k-block per pipeline stage, larger ones two: both
+    sides of the line, with odd numbers of k-blocks and shared experts in the same launches."""
+    sh = W.scaled(W.QWEN, "stages", d_model=320, n_experts=2, d_ff=192, max_k=1, n_shared=1,
+                  d_ff_shared=192)
+    run_parity(sh, W.make_layer(sh), [T, T])
+
+
 def test_sm_pair_one_large_group():
     """One expert takes every token of a 2100-token call: 8 full SM-pair tiles and a partial one."""
     lw = W.make_layer(OLMOE_S)
