@@ -13,6 +13,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -166,8 +167,9 @@ extern "C" eat_status eat_route_noalloc(const void* x, int32_t T, int32_t d_mode
     const eat_status s = scratch_address(&scratch);
     if (s != EAT_OK) return s;
 
-    int split = eat::router_split(T, d_model, n_experts);
-    while (split > 1 && (size_t)split * T * n_experts > kScratchScores) split /= 2;
+    // as many slices of d as the scratch holds
+    const int split = std::min<int>(eat::router_split(T, d_model, n_experts),
+                                    (int)(kScratchScores / ((size_t)T * n_experts)));
     e = eat::launch_router_logits(x, xdtype == EAT_BF16, w_router, T, d_model, n_experts, split,
                                   scratch, st);
     if (e == cudaSuccess)
