@@ -508,6 +508,14 @@ eat_status eat_create(const eat_layer_desc* desc, const eat_params* params, eat_
     h->opart_rows = tc_opart_rows(h->tc);
   }
 
+  if (h->backend == 0) {
+    const cudaError_t ce = simt_configure();
+    if (ce != cudaSuccess) {
+      free_handle(h);
+      return fail(nullptr, EAT_ERR_CUDA, std::string("fp32 kernels: ") + cudaGetErrorString(ce));
+    }
+  }
+
   // (the split depends on the call's number of 64-token tiles, so the largest T of each counts)
   int max_lsplit = 0;
   for (int T0 = 0; T0 < h->Tmax; T0 += kRouterTileT) {

@@ -183,6 +183,9 @@ struct GroupMap {
 // tokens and K selections (or shared experts) of width F; each shape has its own row tiles.
 enum class SimtShape { kSmall, kMid, kLarge };
 SimtShape simt_shape(int T, int K, int F);
+// Lets the kernels use their shared memory on the current device (eat_create, so that it holds for
+// the device of every handle).
+cudaError_t simt_configure();
 constexpr int simt_rows_up(SimtShape s) {
   return s == SimtShape::kLarge ? 64 : s == SimtShape::kMid ? 32 : 16;
 }

@@ -22,8 +22,6 @@
 // and down 26.6 + 46.1 us at 64 tokens, 108 + 95 us at 1999.)
 #include "eat_internal.cuh"
 
-#include <mutex>
-
 namespace eat {
 
 namespace {
@@ -265,15 +263,14 @@ ffn_simt_kernel(const float* __restrict__ in, const float* __restrict__ w0,
 }
 
 template <class C>
+cudaError_t configure_simt() {
+  return cudaFuncSetAttribute(ffn_simt_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              C::SMEM);
+}
+
+template <class C>
 cudaError_t launch_simt(const float* in, const float* w0, const float* w1, int Fout, int Kdim,
                         const GroupMap& gm, float* out, cudaStream_t st) {
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(ffn_simt_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    C::SMEM);
-  });
-  if (attr_err != cudaSuccess) return attr_err;
   const dim3 grid((Fout + C::FEAT - 1) / C::FEAT, gm.max_tiles);
   if (grid.y == 0) return cudaSuccess;
   return launch_pdl(ffn_simt_kernel<C>, grid, dim3(C::THREADS), C::SMEM, st, in, w0, w1, Fout,
@@ -281,6 +278,16 @@ cudaError_t launch_simt(const float* in, const float* w0, const float* w1, int F
 }
 
 }  // namespace
+
+cudaError_t simt_configure() {
+  cudaError_t e = configure_simt<SimtLargeUp>();
+  if (e == cudaSuccess) e = configure_simt<SimtLargeDown>();
+  if (e == cudaSuccess) e = configure_simt<SimtMidUp>();
+  if (e == cudaSuccess) e = configure_simt<SimtMidDown>();
+  if (e == cudaSuccess) e = configure_simt<SimtSmallUp>();
+  if (e == cudaSuccess) e = configure_simt<SimtSmallDown>();
+  return e;
+}
 
 SimtShape simt_shape(int T, int K, int F) {
   // selected rows x width: the lines of the table at the top of this file (512 and 1999 tokens)

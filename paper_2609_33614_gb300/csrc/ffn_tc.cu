@@ -1361,7 +1361,8 @@ bool encode_gu4(CUtensorMap* m, const void* gate, const void* up, long long rows
   cuuint32_t box[4] = {(cuuint32_t)(e4m3 ? kBK8 : kBK), 16, 2, 4};  // 128 bytes of each row
   cuuint32_t estr[4] = {1, 1, 1, 1};
   const bool ok = fn(m, e4m3 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
-                     const_cast<char*>(lo), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                     const_cast<char*>(lo), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
   *gate_first = gf;
