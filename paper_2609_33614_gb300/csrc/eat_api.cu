@@ -268,9 +268,7 @@ eat_status run_shared(eat_handle* h, const TcCall& c, const void* x, int T, cuda
 // and keep them in the call's stream after the routed experts.
 bool shared_on_side_stream(const eat_handle* h, int T, int tile_rows) {
   if (h->S == 0 || h->backend != 1) return false;
-  const long long units =
-      (long long)h->S * ((h->Fs + 127) / 128) * ((T + tile_rows - 1) / tile_rows);
-  return units < h->tc.num_sms;
+  return tc_shared_beside(h->tc, T, tile_rows);
 }
 
 // x_host (or null): see run_route; the caller has checked that the router copies x for this call

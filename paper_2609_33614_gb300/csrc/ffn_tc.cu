@@ -5,8 +5,9 @@
 //
 // Orientation ("swap AB"): a tile is 128 weight rows (output features of one expert) x BN tokens
 // (16..128 rows of that expert's slot list), so decode calls with a handful of tokens still issue
-// full M = 128 MMAs and simply stream the activated experts' weights.  Calls of 512 tokens or more
-// run on SM pairs instead (tc_pair_kernel below: M = 256 weight rows x 256 tokens per MMA).
+// full M = 128 MMAs and simply stream the activated experts' weights.  Calls of 512 tokens or more,
+// and some from 129 on (tc_tile_rows), run on SM pairs instead (tc_pair_kernel below: M = 256 weight
+// rows x 256 tokens per MMA).
 //   gate/up kernel: D_gate = Wg[e, f0:f0+128, :] . Xperm[slots]^T and D_up likewise, both in TMEM;
 //       the epilogue writes act[slot, f] = silu(D_gate) * D_up in bf16 (fp32 accumulation).
 //   down kernel:    D = Wd[e, c0:c0+128, :] . act[slots]^T over a K slice: with split-K (decode)
@@ -1506,13 +1507,25 @@ cudaError_t launch_bn(int bn, const CUtensorMap& a0, const CUtensorMap& a1, cons
 // 234 / 203; DeepSeek-V2-Lite 333 (31) 209 / 223, 600 (56) 231 / 233, 1000 300 / 265.  (On a single
 // SM the interleaved 256-token gate/up moves the same shared-memory bytes per flop as two 128-token
 // accumulators and measured slower: OLMoE prefill gate/up 294 -> 316 us.)
+//   So do calls of more than 128 tokens whose shared experts would have too many 128-token units to
+// run beside the routing: on pairs they either have few enough again or follow the routed units in the
+// same launches, where the single-SM kernels give them launches of their own.  Single SM / pairs:
+// Qwen 385 tokens 172 / 142, 450 179 / 150, 511 176 / 160; with shared experts twice as wide 129
+// 139 / 111, 257 163 / 149, 384 187 / 164; one shared expert of 8192 features (128 experts, K = 1) 257
+// 129 / 95.  64 experts with K = 8 and two shared experts of 5632 lose in a part of their range: 200
+// 184 / 166, 333 202 / 217, 500 232 / 207.
 constexpr int kPairMinTokens = 512, kPairMinRows = 64;
+bool tc_shared_beside(const TcLayer& L, int T, int tile_rows) {
+  const long long units =
+      (long long)L.S * ((L.Fs + kBM - 1) / kBM) * ((T + tile_rows - 1) / tile_rows);
+  return units < L.num_sms;
+}
 int tc_tile_rows(const TcLayer& L, int T) {
   for (int i = 0; i < kNumBN - 1; ++i)
     if (T <= kBNs[i]) return kBNs[i];
-  const bool pair = T >= kPairMinTokens || (T > kBNs[kNumBN - 1] &&
-                                            (long long)T * L.K >= (long long)kPairMinRows * L.E);
-  return pair && !L.w8 ? kPairBN : kBNs[kNumBN - 1];
+  const bool pair = T >= kPairMinTokens || (long long)T * L.K >= (long long)kPairMinRows * L.E ||
+                    (L.S > 0 && !tc_shared_beside(L, T, kBNs[kNumBN - 1]));
+  return pair && T > kBNs[kNumBN - 1] && !L.w8 ? kPairBN : kBNs[kNumBN - 1];
 }
 // bf16 calls whose tokens fit one tile read the token rows themselves as the gate/up kernel's B tile
 // (tc_ffn_kernel's TOK), so nothing is gathered; larger calls copy their rows to slot order first,

@@ -58,6 +58,8 @@ int tc_bind(TcLayer& L, const eat_layer_desc& D, void* xperm, void* act, void* s
             const TcWork& q, const char** msg);
 void tc_destroy(TcLayer& L);
 int tc_tile_rows(const TcLayer& L, int T);       // gate/up token rows per tile, call of T tokens
+// The shared experts' GEMMs of the call have fewer work units than the GPU has SMs.
+bool tc_shared_beside(const TcLayer& L, int T, int tile_rows);
 int tc_tile_rows_down(const TcLayer& L, int T);  // down-projection token rows per tile
 // The call's gate/up reads its token rows in token order (no row is copied to slot order).
 bool tc_token_tiles(const TcLayer& L, int T);

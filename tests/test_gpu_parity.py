@@ -427,6 +427,16 @@ def test_sm_pair_smallest_calls(E, K, S, T):
     run_parity(sh, W.make_layer(sh), [T, T - 1])
 
 
+@pytest.mark.parametrize("S,Fs,T", [(4, 1408, 385), (2, 4864, 129), (1, 9728, 300)])
+def test_sm_pair_calls_of_large_shared_experts(S, Fs, T):
+    """bf16 calls above 128 tokens whose shared experts have a unit of 128 features and 128 tokens for
+    each SM run on SM pairs, beside the routing (385, 129) or in the routed launches (300); 385 and
+    129 tokens are the first such calls, and one token less is still on single SMs."""
+    sh = W.scaled(W.QWEN, "pairshared", d_model=256, n_experts=64, d_ff=192, max_k=4, n_shared=S,
+                  d_ff_shared=Fs)
+    run_parity(sh, W.make_layer(sh), [T, T - 1])
+
+
 @pytest.mark.parametrize("T", [1000, 1100])
 def test_sm_pair_stage_sizes(T):
     """Calls of at most 512 rows per expert run one k-block per pipeline stage, larger ones two: both
