@@ -733,10 +733,15 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
 constexpr int kPairBN = 256;
 constexpr int kPairRows = kPairBN / 2;
 
-// W8 (fp8 layers): the tile is 128 tokens; CTA 0 holds their hi rows of B and CTA 1 their lo rows, so
-// one MMA of N = 2 n multiplies the A tile with both (accumulator columns [0, n) and [n, 2 n), added
-// in the epilogue, n the unit's rows rounded up to 16) and each CTA stages 32 KB per 128-element
-// k-block where the single-SM kernel stages 48 (down) or 64 KB (gate/up) for the same MMAs.
+// W8 (fp8 layers): the tile is 128 tokens, and each CTA stages 32 KB per 128-element k-block where
+// the single-SM kernel stages 48 (down) or 64 KB (gate/up) for the same MMAs.  The sums are those of
+// the single-SM kernel's 128-token tiles, bit for bit, so a call's results do not depend on which of
+// the two runs it (a gate/up whose weights have no 4D view stays on single SMs):
+//   gate/up: each CTA holds the hi and the lo rows of half of the tokens; every k-step issues W . hi
+//       and then W . lo into the same accumulator;
+//   down: CTA 0 holds the tokens' hi rows and CTA 1 their lo rows, so one MMA of N = 2 n multiplies
+//       the A tile with both (accumulator columns [0, n) and [n, 2 n), added in the epilogue, n the
+//       unit's rows rounded up to 16).
 template <int MODE, bool IL4 = false, bool W8 = false, int KPS = 2>
 struct PairCfg {
   static constexpr int kBN = W8 ? kPairRows : kPairBN;  // token rows of a unit
@@ -957,8 +962,9 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         const int a_rows = sh ? args_s.a_rows_per_group : args.a_rows_per_group;
         const int b_shift = sh ? args_s.b_shift_per_group : args.b_shift_per_group;
         const int a_row = w.g * a_rows + w.m0 + (int)rank * C::kFeat;
-        // (fp8: this CTA's plane of the tokens' rows)
-        const int b_row = w.slot0 - w.g * b_shift + (int)rank * (W8 ? args.b_lo_rows : n / 2);
+        // this CTA's half of the tokens; of an fp8 down unit: its plane of all of them
+        const int b_row =
+            w.slot0 - w.g * b_shift + (int)rank * (W8 && !IL ? args.b_lo_rows : n / 2);
         for (int kb = w.kb0; kb < w.kb1; kb += C::kKPS) {
           const int nk = min(C::kKPS, w.kb1 - kb);  // k-blocks of this stage
           if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, args.err, 1u, true)) {
@@ -982,6 +988,9 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 tma_load_2d_pair(sj, mA0, fb, kx, a_row);
               }
               tma_load_2d_pair(sj + C::kABytes, mB, fb, kx, b_row);
+              if (W8 && IL)
+                tma_load_2d_pair(sj + C::kABytes + C::kBBytes / 2, mB, fb, kx,
+                                 b_row + args.b_lo_rows);
             }
           }
           ++issued;
@@ -1016,8 +1025,9 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         }
         tc_fence_after();
         const uint32_t d0 = tmem_base + (uint32_t)(buf * C::kAccCols);
-        const uint32_t idesc = W8 ? idesc_e4m3_pair(2 * pair_n8(w.nrows))
-                                  : idesc_bf16_pair(pair_n(w.nrows));
+        const uint32_t idesc = !W8  ? idesc_bf16_pair(pair_n(w.nrows))
+                               : IL ? idesc_e4m3_pair(pair_n(w.nrows))
+                                    : idesc_e4m3_pair(2 * pair_n8(w.nrows));
         for (int kb = w.kb0; kb < w.kb1; kb += C::kKPS) {
           const int nk = min(C::kKPS, w.kb1 - kb);
           if (!mbar_wait(&full[stage], phase, abort_flag, args.err, 8u, true)) {
@@ -1030,11 +1040,14 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             if (j < nk) {
               const uint32_t sa = smem_u32(smem + stage * C::kStageBytes + j * C::kSubBytes);
               const uint64_t da = sdesc_k128(sa), db = sdesc_k128(sa + C::kABytes);
+              const uint64_t dl = sdesc_k128(sa + C::kABytes + C::kBBytes / 2);  // fp8 gate/up
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
                 const uint32_t acc = (kb > w.kb0 || j > 0 || k > 0) ? 1u : 0u;
                 if (W8) mma_e4m3_pair(d0, sdesc_step(da, k), sdesc_step(db, k), idesc, acc);
                 else mma_bf16_pair(d0, sdesc_step(da, k), sdesc_step(db, k), idesc, acc);
+                if (W8 && IL)
+                  mma_e4m3_pair(d0, sdesc_step(da, k), sdesc_step(dl, k), idesc, 1u);
               }
             }
           }
@@ -1076,8 +1089,11 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * C::kAccCols);
       const int f = w.m0 + (int)rank * C::kFeat + 16 * q + (lane & 15);
       const bool fok = f < M;
-      float rs = 1.0f;  // fp8: the scale of this lane's weight row
-      if (W8 && fok) rs = (mine_is_gate ? args.scale0 : args.scale1)[(size_t)w.g * M + f];
+      float sg = 1.0f, su = 1.0f;  // fp8: the scales of the feature's gate and up weight rows
+      if (W8 && fok) {
+        sg = args.scale0[(size_t)w.g * M + f];
+        su = args.scale1[(size_t)w.g * M + f];
+      }
       const float* bsc = W8 ? args.bscale + (w.slot0 - w.g * args.b_shift_per_group) : nullptr;
       constexpr int kCols = BN / 2;  // token columns of one warp
       const int c_end = min(kCols * ch + kCols, w.nrows);
@@ -1085,17 +1101,6 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
         uint32_t v0[16], v1[16];
         tmem_ld16(tbase + c0, v0);
         tmem_ld16(tbase + c0 + 16, v1);
-        if constexpr (W8) {  // + the lo parts' columns, times the weight row's scale
-          uint32_t l0[16], l1[16];
-          tmem_ld16(tbase + pair_n8(w.nrows) + c0, l0);
-          tmem_ld16(tbase + pair_n8(w.nrows) + c0 + 16, l1);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            v0[j] = __float_as_uint((__uint_as_float(v0[j]) + __uint_as_float(l0[j])) * rs);
-            v1[j] = __float_as_uint((__uint_as_float(v1[j]) + __uint_as_float(l1[j])) * rs);
-          }
-        }
         tmem_wait_ld();
         const int cb = c0 + (lo ? 0 : 16);
 #pragma unroll
@@ -1108,8 +1113,8 @@ tc_pair_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
           if (fok && cb + j < w.nrows) {
             if (W8) {
               const float sc = bsc[cb + j];
-              g *= sc;
-              up *= sc;
+              g *= sg * sc;
+              up *= su * sc;
             }
             out[(size_t)(w.slot0 + cb + j) * M + f] = __float2bfloat16_rn(silu_f(g) * up);
           }
@@ -1541,8 +1546,9 @@ bool tc_token_tiles(const TcLayer& L, int T) { return T <= kBNs[kNumBN - 1] && !
 static int streams_weights(int T) { return T <= kBNs[kNumBN - 1] ? 1 : 0; }
 
 // fp8 calls on SM pairs (128-token tiles): every call whose tokens do not fit one tile.  us per
-// call, single SM / pairs: OLMoE 200 tokens 90.7 / 87.1, 3001 379.5 / 364.6, Mixtral shape 400 385.3
-// / 358.6, 1000 660.7 / 620.7, Qwen 333 105.9 / 101.9, DeepSeek-V2-Lite 600 170.0 / 169.8.
+// call, single SM / pairs: OLMoE 130 tokens 80.1 / 79.5, 200 87.3 / 84.8, 3001 383.7 / 372.3, Mixtral
+// shape 333 352.4 / 330.5, 1000 663.9 / 627.5, Qwen 333 107.1 / 105.3, DeepSeek-V2-Lite 600 175.9 /
+// 174.0.
 static bool pairs8(const TcLayer& L, int T) { return L.w8 && T > kBNs[kNumBN - 1]; }
 
 // bf16 SM pairs: one k-block per stage for calls of at most 512 rows per expert on average.  us per
@@ -1766,7 +1772,7 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     if (shared) {
       shared_args(a);
       a.gate_first = m->sgate_first ? 1 : 0;
-      return launch_pair8<kModeGateUpIL>(m->wsgu4, m->xqt[bn_index(kPairRows)], a,
+      return launch_pair8<kModeGateUpIL>(m->wsgu4, m->xqt[bn_index(kPairRows / 2)], a,
                                          (long long)L.S * ((c.T + bn - 1) / bn) * a.m_tiles,
                                          L.num_sms, st);
     }
@@ -1775,7 +1781,7 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     a.row_offs = c.offs;
     a.tile_offs = c.tile_offs;
     a.out = c.act;
-    return launch_pair8<kModeGateUpIL>(m->wgu4, m->xq[bn_index(kPairRows)], a,
+    return launch_pair8<kModeGateUpIL>(m->wgu4, m->xq[bn_index(kPairRows / 2)], a,
                                        ((long long)(c.T * L.K + bn - 1) / bn + L.E) * a.m_tiles,
                                        L.num_sms, st);
   }

@@ -456,8 +456,7 @@ def test_sm_pair_one_large_group():
 
 @pytest.mark.parametrize("E,K,T", [(256, 8, 1500), (64, 2, 1100)])
 def test_fp8_large_calls_small_groups(E, K, T):
-    """e4m3 weights at call sizes where bf16 layers switch to the SM-pair kernels (fp8 layers keep
-    the single-SM kernels, 128-token tiles): mostly partial tiles."""
+    """e4m3 weights, large calls of many experts: mostly partial 128-token tiles."""
     sh = W.scaled(W.OLMOE, f"pair8-{E}", d_model=256, n_experts=E, d_ff=384, max_k=K)
     lw8 = W.to_fp8(W.make_layer(sh))
     layer = eat.EatLayer.from_workload(lw8, T, gpu_params(sh))
@@ -470,14 +469,43 @@ def test_fp8_large_calls_small_groups(E, K, T):
     (256, 1024, 64, 4, 0, [130, 700]),  # mostly partial tiles, down projections split along K
 ])
 def test_fp8_sm_pairs(d, F, E, K, S, Ts):
-    """e4m3 layers on SM pairs (calls above 128 tokens): the hi rows in one CTA, the lo rows in the
-    other, 128-token tiles of every width."""
+    """e4m3 layers on SM pairs (calls above 128 tokens): 128-token tiles of every width."""
     sh = W.scaled(W.QWEN if S else W.OLMOE, f"p8-{d}", d_model=d, n_experts=E, d_ff=F, max_k=K,
                   n_shared=S, d_ff_shared=F if S else 0)
     lw8 = W.to_fp8(W.make_layer(sh))
     layer = eat.EatLayer.from_workload(lw8, max(Ts), gpu_params(sh))
     run_parity(sh, lw8.dequantized(), Ts, layer=layer)
     layer.close()
+
+
+@pytest.mark.parametrize("d,F,E,K,S,Ts", [
+    (192, 320, 6, 2, 2, [129, 300]),    # ragged last k-blocks, partial feature tiles, shared experts
+    (256, 1024, 64, 4, 0, [130, 700]),  # mostly partial tiles
+    (2048, 512, 4, 2, 1, [600]),        # full tiles
+])
+def test_fp8_results_do_not_depend_on_the_weights_addresses(d, F, E, K, S, Ts):
+    """The SM-pair gate/up of an e4m3 layer needs one 4D view over its gate and up weights; without
+    it (here: gate and up are one tensor) the call runs on single SMs.  Equal weights, equal bits."""
+    sh = W.scaled(W.QWEN if S else W.OLMOE, f"p8a-{d}", d_model=d, n_experts=E, d_ff=F, max_k=K,
+                  n_shared=S, d_ff_shared=F if S else 0)
+    lw = W.make_layer(sh)
+    lw.w_up, lw.ws_up = lw.w_gate, lw.ws_gate
+    lw8 = W.to_fp8(lw)
+    t = {n: v.cuda() for n, v in vars(lw8).items() if isinstance(v, torch.Tensor)}
+    sc = {n: v.cuda() for n, v in lw8.scales.items()}
+
+    def layer(up, ws_up):
+        return eat.EatLayer(t["w_router"], t["b_router"], t["w_gate"], up, t["w_down"], max(Ts),
+                            gpu_params(sh), t.get("ws_gate"), ws_up, t.get("ws_down"), scales=sc)
+    A = layer(t["w_gate"], t.get("ws_gate"))
+    B = layer(t["w_gate"].clone(), t["ws_gate"].clone() if S else None)
+    for T in Ts:
+        x = W.make_tokens(sh, T, step=T).cuda()
+        assert torch.equal(A.forward(x, 0), B.forward(x, 0))
+    for u, v in zip(A.accounts(), B.accounts()):
+        assert torch.equal(u, v)
+    A.close()
+    B.close()
 
 
 def test_fp8_large_call_one_group():
