@@ -199,10 +199,10 @@ eat_status check_call(eat_handle* h, const void* x, int32_t T, int32_t ppl_sign)
   return check_state(h);
 }
 
-// Router + selection into (idx, w, k, psel).  x_host (or null): the router kernel reads the
+// Router + selection into (idx, w, k, psel), and into the caller's copies.  x_host (or null): the router kernel reads the
 // tokens there (a page-locked host buffer) and writes them to x, which later kernels read.
 eat_status run_route(eat_handle* h, const void* x, int T, int ppl_sign, int32_t* idx, float* w,
-                     int32_t* k, float* psel, bool write_tau, cudaStream_t st,
+                     int32_t* k, float* psel, RouteCopies copies, bool write_tau, cudaStream_t st,
                      const void* x_host = nullptr) {
   RouteParams rp = route_params(h->prm, ppl_sign);
   rp.opd_scale = h->desc.opd_scale;
@@ -215,7 +215,7 @@ eat_status run_route(eat_handle* h, const void* x, int T, int ppl_sign, int32_t*
   if (route_fused(xr, h->bf16, h->desc.w_router, T, h->d, h->E))
     return launch(h, kRoute, st, "route", [&] {
       return launch_route_fused(xr, h->bf16, h->desc.w_router, h->desc.b_router, T, h->d, h->E,
-                                h->K, h->N, h->P, h->C, rp, idx, w, k, psel, st,
+                                h->K, h->N, h->P, h->C, rp, idx, w, k, psel, copies, st,
                                 x_host ? const_cast<void*>(x) : nullptr);
     });
   const int split = router_split(T, h->d, h->E);
@@ -228,7 +228,7 @@ eat_status run_route(eat_handle* h, const void* x, int T, int ppl_sign, int32_t*
   }));
   EAT_TRY(launch(h, kSelect, st, "route select", [&] {
     return launch_route_select(h->logit_part, split, h->desc.b_router, T, h->E, h->K, h->N,
-                               h->P, h->C, rp, idx, w, k, psel, st);
+                               h->P, h->C, rp, idx, w, k, psel, copies, st);
   }));
   return EAT_OK;
 }
@@ -308,17 +308,16 @@ eat_status run_forward(eat_handle* h, const void* x, int T, int ppl_sign, void* 
     e = cudaEventRecord(h->ev_join, h->side_st);
     if (e != cudaSuccess) return cuda_fail(h, e, "shared-expert stream join");
   }
-  // the caller's routing buffers take the place of the handle's (the later kernels read them; a
-  // pointer that is not aligned to its elements gets a copy at the end): three copies behind the
-  // call, which programmatic launches cannot overlap, cost an OLMoE decode call 12 of 67 us
-  auto own = [](const void* p) { return !p || ((uintptr_t)p & 3) != 0; };
-  int32_t* const idx = own(idx_opt) ? h->idx : idx_opt;
-  float* const w = own(w_opt) ? h->w : w_opt;
-  int32_t* const k = own(k_opt) ? h->k : k_opt;
+  // the selection writes the caller's routing buffers beside the handle's (a pointer that is not
+  // aligned to its elements gets a copy at the end): three copies behind the call, which
+  // programmatic launches cannot overlap, cost an OLMoE decode call 12 of 67 us.  No kernel of the
+  // call reads the caller's buffers, whose contents another call may change meanwhile.
+  auto direct = [](auto* p) { return ((uintptr_t)p & 3) == 0 ? p : nullptr; };
+  const RouteCopies copies{direct(idx_opt), direct(w_opt), direct(k_opt)};
   if (x_host && side) return fail(h, EAT_ERR_UNSUPPORTED, "host-read input with side-stream experts");
-  EAT_TRY(run_route(h, x, T, ppl_sign, idx, w, k, h->psel, true, st, x_host));
+  EAT_TRY(run_route(h, x, T, ppl_sign, h->idx, h->w, h->k, h->psel, copies, true, st, x_host));
   EAT_TRY(launch(h, kPermute, st, "permute", [&] {
-    return launch_permute(idx, h->psel, T, h->K, h->E, tile_rows, tile_rows_down,
+    return launch_permute(h->idx, h->psel, T, h->K, h->E, tile_rows, tile_rows_down,
                           h->perm, h->chunk_cnt, st);
   }));
   const int rows = T * h->K;
@@ -364,23 +363,21 @@ eat_status run_forward(eat_handle* h, const void* x, int T, int ppl_sign, void* 
   EAT_TRY(launch(h, kCombine, st, "combine", [&] {
     const int tc = h->backend == 1;
     return launch_combine(h->bf16, h->opart, tc && n_split == 1, n_split, rows, h->perm.slot_of,
-                          w, h->sout, tc, h->S, T, h->K, h->d, y, h->nrm_part, h->status, st);
+                          h->w, h->sout, tc, h->S, T, h->K, h->d, y, h->nrm_part, h->status, st);
   }));
   EAT_TRY(launch(h, kAccount, st, "account update", [&] {
     return launch_account(h->perm.offs, h->perm.perm_p, h->nrm_part, h->nb, h->E, T, rows,
                           h->prm.alpha, h->N, h->P, h->C, h->st_n, h->st_p, h->st_norm,
                           h->counters, h->acc_sums, h->acc_tickets, h->status, h->mirror_dev, st);
   }));
-  if ((idx_opt && idx != idx_opt) || (w_opt && w != w_opt) || (k_opt && k != k_opt)) {
-    cudaError_t e = cudaSuccess;
-    if (idx_opt && idx != idx_opt && e == cudaSuccess)
-      e = cudaMemcpyAsync(idx_opt, h->idx, sizeof(int32_t) * rows, cudaMemcpyDeviceToDevice, st);
-    if (w_opt && w != w_opt && e == cudaSuccess)
-      e = cudaMemcpyAsync(w_opt, h->w, sizeof(float) * rows, cudaMemcpyDeviceToDevice, st);
-    if (k_opt && k != k_opt && e == cudaSuccess)
-      e = cudaMemcpyAsync(k_opt, h->k, sizeof(int32_t) * T, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_fail(h, e, "routing copy-out");
-  }
+  cudaError_t e = cudaSuccess;
+  if (idx_opt != copies.idx)
+    e = cudaMemcpyAsync(idx_opt, h->idx, sizeof(int32_t) * rows, cudaMemcpyDeviceToDevice, st);
+  if (w_opt != copies.w && e == cudaSuccess)
+    e = cudaMemcpyAsync(w_opt, h->w, sizeof(float) * rows, cudaMemcpyDeviceToDevice, st);
+  if (k_opt != copies.k && e == cudaSuccess)
+    e = cudaMemcpyAsync(k_opt, h->k, sizeof(int32_t) * T, cudaMemcpyDeviceToDevice, st);
+  if (e != cudaSuccess) return cuda_fail(h, e, "routing copy-out");
   return EAT_OK;
 }
 
@@ -649,7 +646,7 @@ eat_status eat_route(eat_handle* h, const void* x, int32_t T, int32_t ppl_sign, 
                      float* w, int32_t* k, void* stream) {
   EAT_TRY(check_call(h, x, T, ppl_sign));
   if (!idx || !w || !k) return fail(h, EAT_ERR_INVALID_ARG, "idx, w and k must be non-NULL");
-  return run_route(h, x, T, ppl_sign, idx, w, k, nullptr, false, (cudaStream_t)stream);
+  return run_route(h, x, T, ppl_sign, idx, w, k, nullptr, {}, false, (cudaStream_t)stream);
 }
 
 eat_status eat_moe_forward(eat_handle* h, const void* x, int32_t T, int32_t ppl_sign, void* y,

@@ -121,6 +121,13 @@ cudaError_t launch_router_logits(const void* x, int x_bf16, const float* w_route
                                  int E, int n_split, float2* part, cudaStream_t st,
                                  void* xcopy = nullptr);
 bool router_copies_x(const void* x, int x_bf16, const float* w_router, int T, int d, int E);
+// The caller's copies of a selection's outputs (each or all null).  They are written beside the
+// selection's own outputs, which alone the later kernels of a call read.
+struct RouteCopies {
+  int32_t* idx = nullptr;
+  float* w = nullptr;
+  int32_t* k = nullptr;
+};
 // Scores and selection in one launch, without scratch, for the calls for which route_fused holds
 // (x, w_router: their alignment); xcopy as above.
 bool route_fused(const void* x, int x_bf16, const float* w_router, int T, int d, int E);
@@ -128,13 +135,13 @@ cudaError_t launch_route_fused(const void* x, int x_bf16, const float* w_router,
                                const float* b_router, int T, int d, int E, int K,
                                const int64_t* accN, const double* accP, const double* accC,
                                RouteParams rp, int32_t* idx, float* w, int32_t* k, float* psel,
-                               cudaStream_t st, void* xcopy = nullptr);
+                               RouteCopies copies, cudaStream_t st, void* xcopy = nullptr);
 // Warp-per-token softmax + history score + threshold + selection + renormalisation; the router
 // scores are the sum over the n_split slices of part ([split][T][E] fp32 pairs).
 cudaError_t launch_route_select(const float2* part, int n_split, const float* b_router, int T,
                                 int E, int K, const int64_t* accN, const double* accP,
                                 const double* accC, RouteParams rp, int32_t* idx, float* w,
-                                int32_t* k, float* psel, cudaStream_t st);
+                                int32_t* k, float* psel, RouteCopies copies, cudaStream_t st);
 constexpr int kRouterTileT = 64;    // tokens of a tile of the larger calls' routers
 constexpr int kSmallRouterT = 128;  // calls up to this many tokens use the GEMV-style router
 int router_split(int T, int d, int E);

@@ -539,6 +539,7 @@ struct SelectArgs {
   float* out_w;
   int32_t* out_k;
   float* out_p;
+  RouteCopies copies;
 };
 
 // One warp: the selection of token t from its router scores x . w_r (compensated pairs hi, lo of
@@ -742,9 +743,12 @@ __device__ __forceinline__ void select_token(int t, float (&hi)[EPL], float (&lo
     const unsigned b = __ballot_sync(full, sel[i]);
     if (sel[i]) {
       const int pos = base + __popc(b & lt);
+      const float g = p[i] / denom;
       a.out_idx[row + pos] = lane + 32 * i;
-      a.out_w[row + pos] = p[i] / denom;
+      a.out_w[row + pos] = g;
       if (a.out_p) a.out_p[row + pos] = p[i];
+      if (a.copies.idx) a.copies.idx[row + pos] = lane + 32 * i;
+      if (a.copies.w) a.copies.w[row + pos] = g;
     }
     base += __popc(b);
   }
@@ -752,8 +756,13 @@ __device__ __forceinline__ void select_token(int t, float (&hi)[EPL], float (&lo
     a.out_idx[row + lane] = -1;
     a.out_w[row + lane] = 0.f;
     if (a.out_p) a.out_p[row + lane] = 0.f;
+    if (a.copies.idx) a.copies.idx[row + lane] = -1;
+    if (a.copies.w) a.copies.w[row + lane] = 0.f;
   }
-  if (lane == 0) a.out_k[t] = base;
+  if (lane == 0) {
+    a.out_k[t] = base;
+    if (a.copies.k) a.copies.k[t] = base;
+  }
 }
 
 template <int EPL>
@@ -1104,18 +1113,20 @@ cudaError_t launch_router_logits(const void* x, int x_bf16, const float* w_route
 
 static SelectArgs select_args(const float* b_router, int T, int E, int K, const int64_t* accN,
                               const double* accP, const double* accC, const RouteParams& rp,
-                              int32_t* idx, float* w, int32_t* k, float* psel) {
+                              int32_t* idx, float* w, int32_t* k, float* psel,
+                              RouteCopies copies) {
   return SelectArgs{b_router, T, E, K, accN, accP, accC, rp,
-                    (float)(1.0 / (double)rp.temperature), idx, w, k, psel};
+                    (float)(1.0 / (double)rp.temperature), idx, w, k, psel, copies};
 }
 
 cudaError_t launch_route_select(const float2* part, int n_split, const float* b_router, int T,
                                 int E, int K, const int64_t* accN, const double* accP,
                                 const double* accC, RouteParams rp, int32_t* idx, float* w,
-                                int32_t* k, float* psel, cudaStream_t st) {
+                                int32_t* k, float* psel, RouteCopies copies, cudaStream_t st) {
   const int warps = kSelectThreads / 32;
   dim3 grid((T + warps - 1) / warps);
-  const SelectArgs a = select_args(b_router, T, E, K, accN, accP, accC, rp, idx, w, k, psel);
+  const SelectArgs a =
+      select_args(b_router, T, E, K, accN, accP, accC, rp, idx, w, k, psel, copies);
 #define EAT_SELECT(EPL) \
   launch_pdl(route_select_kernel<EPL>, grid, dim3(kSelectThreads), 0, st, part, n_split, a)
   if (E <= 32) return EAT_SELECT(1);
@@ -1152,10 +1163,11 @@ cudaError_t launch_route_fused(const void* x, int x_bf16, const float* w_router,
                                const float* b_router, int T, int d, int E, int K,
                                const int64_t* accN, const double* accP, const double* accC,
                                RouteParams rp, int32_t* idx, float* w, int32_t* k, float* psel,
-                               cudaStream_t st, void* xcopy) {
+                               RouteCopies copies, cudaStream_t st, void* xcopy) {
   if (!route_fused(x, x_bf16, w_router, T, d, E) || ((uintptr_t)xcopy & 15) != 0)
     return cudaErrorInvalidValue;
-  const SelectArgs a = select_args(b_router, T, E, K, accN, accP, accC, rp, idx, w, k, psel);
+  const SelectArgs a =
+      select_args(b_router, T, E, K, accN, accP, accC, rp, idx, w, k, psel, copies);
   if (x_bf16)
     return launch_fused_x((const __nv_bfloat16*)x, w_router, d, a, (__nv_bfloat16*)xcopy, st);
   return launch_fused_x((const float*)x, w_router, d, a, (float*)xcopy, st);

@@ -161,7 +161,7 @@ extern "C" eat_status eat_route_noalloc(const void* x, int32_t T, int32_t d_mode
   cudaError_t e;
   if (eat::route_fused(x, xdtype == EAT_BF16, w_router, T, d_model, n_experts)) {
     e = eat::launch_route_fused(x, xdtype == EAT_BF16, w_router, b_router, T, d_model, n_experts,
-                                p.max_k, N, P, C, rp, idx, w, k, nullptr, st);
+                                p.max_k, N, P, C, rp, idx, w, k, nullptr, {}, st);
   } else {
     float2* scratch = nullptr;
     const eat_status s = scratch_address(&scratch);
@@ -174,7 +174,7 @@ extern "C" eat_status eat_route_noalloc(const void* x, int32_t T, int32_t d_mode
                                   scratch, st);
     if (e == cudaSuccess)
       e = eat::launch_route_select(scratch, split, b_router, T, n_experts, p.max_k, N, P, C, rp,
-                                   idx, w, k, nullptr, st);
+                                   idx, w, k, nullptr, {}, st);
   }
   if (e != cudaSuccess) {
     eat::set_thread_error((std::string("eat_route_noalloc launch: ") + cudaGetErrorString(e))

@@ -379,6 +379,48 @@ def test_routing_and_account_outputs(which):
     B.close()
 
 
+@pytest.mark.parametrize("T", [40, 300])
+def test_call_does_not_read_the_callers_routing_buffers(T):
+    """One throw-away buffer for idx, w and k: it ends up with any of them, and the layer's output
+    and accounts are those of a call without routing buffers."""
+    lw = W.make_layer(OLMOE_S)
+    x = W.make_tokens(OLMOE_S, T).cuda()
+    A, B = (eat.EatLayer.from_workload(lw, T, gpu_params(OLMOE_S)) for _ in range(2))
+    buf = torch.empty(T * OLMOE_S.max_k, dtype=torch.int32, device="cuda")
+    y = torch.empty_like(x)
+    for _ in range(2):
+        eat.eat_moe_forward(B.h, x, T, 0, y, buf, buf, buf)
+        assert torch.equal(y, A.forward(x, 0))
+    for u, v in zip(A.accounts(), B.accounts()):
+        assert torch.equal(u, v)
+    A.close()
+    B.close()
+
+
+def test_two_streams_share_throw_away_routing_buffers():
+    """Handles on two streams write their routing into the same buffers: only those are spoiled."""
+    lw = W.make_layer(OLMOE_S)
+    T, n = 64, 20
+    xs = [W.make_tokens(OLMOE_S, T, step=s).cuda() for s in range(2)]
+    layers = [eat.EatLayer.from_workload(lw, T, gpu_params(OLMOE_S)) for _ in range(4)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    idx = torch.empty(T, OLMOE_S.max_k, dtype=torch.int32, device="cuda")
+    w = torch.empty(T, OLMOE_S.max_k, dtype=torch.float32, device="cuda")
+    k = torch.empty(T, dtype=torch.int32, device="cuda")
+    ys = [[torch.empty_like(xs[0]) for _ in range(n)] for _ in range(2)]
+    torch.cuda.synchronize()
+    for i in range(n):
+        for s in range(2):
+            eat.eat_moe_forward(layers[s].h, xs[s], T, 0, ys[s][i], idx, w, k,
+                                stream=streams[s].cuda_stream)
+    torch.cuda.synchronize()
+    for s in range(2):
+        for i in range(n):
+            assert torch.equal(ys[s][i], layers[2 + s].forward(xs[s], 0))
+    for L in layers:
+        L.close()
+
+
 def test_token_tiles_of_small_calls():
     """bf16 gate/up tiles that hold the call's tokens in token order: token counts at and around the
     tile widths, then a non-finite token among others (its column must not reach theirs)."""
