@@ -157,16 +157,18 @@ extern "C" eat_status eat_route_noalloc(const void* x, int32_t T, int32_t d_mode
   rp.ppl_up = (float)p.ppl_up;
   rp.ppl_down = (float)p.ppl_down;
 
+  // looked up by every call, also by those that route in one launch and need no scratch: the first
+  // call of any size is then the one that the header asks to be made before a stream capture
+  float2* scratch = nullptr;
+  const eat_status s = scratch_address(&scratch);
+  if (s != EAT_OK) return s;
+
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e;
   if (eat::route_fused(x, xdtype == EAT_BF16, w_router, T, d_model, n_experts)) {
     e = eat::launch_route_fused(x, xdtype == EAT_BF16, w_router, b_router, T, d_model, n_experts,
                                 p.max_k, N, P, C, rp, idx, w, k, nullptr, {}, st);
   } else {
-    float2* scratch = nullptr;
-    const eat_status s = scratch_address(&scratch);
-    if (s != EAT_OK) return s;
-
     // as many slices of d as the scratch holds
     const int split = std::min<int>(eat::router_split(T, d_model, n_experts),
                                     (int)(kScratchScores / ((size_t)T * n_experts)));

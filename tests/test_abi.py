@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2609_33614_gb300 import build, eat
 
@@ -107,6 +108,21 @@ def test_binding_raises_with_message(lib):
         eat._check(lib.eat_route(None, 1, 1, 0, 1, 1, 1, None))
     assert ei.value.status == eat.EAT_ERR_INVALID_ARG
     assert "null handle" in str(ei.value)
+
+
+@pytest.mark.parametrize("T", [1, 128, 300])
+def test_noalloc_looks_its_scratch_up_in_calls_of_any_size(lib, T):
+    """The first eat_route_noalloc call is the one a program makes before a stream capture, so the
+    look-up belongs to every call, whether it routes in one launch (T <= 128) or uses the scratch:
+    without a device, both stop there."""
+    if torch.cuda.is_available():
+        pytest.skip("the pointers are not device memory")
+    p = eat.eat_default_params(2)
+    a = [4096 * i for i in range(1, 9)]
+    r = lib.eat_route_noalloc(a[0], T, 256, 64, eat.EAT_BF16, a[1], None, a[2], a[3], a[4],
+                              ctypes.byref(p), 0, a[5], a[6], a[7], None)
+    assert r == eat.EAT_ERR_CUDA
+    assert re.match(rb"cudaGetDevice|cudaGetSymbolAddress", lib.eat_last_error(None))
 
 
 def test_layer_policy_and_ppl_argument_checks(lib):

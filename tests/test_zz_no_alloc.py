@@ -70,6 +70,24 @@ def test_noalloc_matches_route_and_oracle_two_calls(layer, calls):
         par.check_routing(routing, par.gpu_selection(idx, k), w.cpu().numpy(), SHAPE.max_k)
 
 
+def test_noalloc_small_call_then_captured_larger_call(layer):
+    """A program warms up with a decode batch (one launch, no scratch) and then captures a call that
+    uses the scratch."""
+    L, _ = layer
+    _noalloc(L, W.make_tokens(SHAPE, 8, step=50).cuda(), 0)
+    x = W.make_tokens(SHAPE, 300, step=51).cuda()
+    N, P, C = L.accounts()
+    idx, w, k = (t.zero_() for t in L.route(x, 0))
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        eat.eat_route_noalloc(x, 300, L.d, L.E, eat.EAT_BF16, L._keep[0], L._keep[1], N, P, C,
+                              L.params, 0, idx, w, k)
+    g.replay()
+    torch.cuda.synchronize()
+    for got, want in zip((idx, w, k), _noalloc(L, x, 0)):
+        assert torch.equal(got, want)
+
+
 def test_noalloc_rejects_batches_beyond_its_scratch(layer):
     L, _ = layer
     T = (1 << 20) // 8 // L.E + 1   # T * E > 131072 router scores
