@@ -1,7 +1,7 @@
 // Router and EAT selection (§3.1-§3.4 of the EAT paper, Eq. 1-8).
 //
-//  route_fused_kernel (T <= 128 and d <= 4096, and some larger calls): scores and selection of a
-//      small call in one launch, a cluster of CTAs per group of tokens.
+//  route_fused_kernel (T <= 128 and d <= 4096, and some larger calls, see route_fused): scores and
+//      selection of a small call in one launch, a cluster of CTAs per group of tokens.
 //  router_logits_small_kernel (T <= 128, d > 4096) / router_logits_sk_kernel (bf16 x, larger calls;
 //      stream-K over tiles and chunks of d) / router_logits_kernel (other large calls; both tiled
 //      through shared memory): partial router scores x . w_r over slices of d: fp32 FMA inside
@@ -819,7 +819,7 @@ route_select_kernel(const float2* __restrict__ part, int n_split, const SelectAr
 // registers are bounded so that three CTAs share an SM (a second wave of clusters of eight took
 // 9.1 us instead of 5.6 at 16 tokens).  us per routing call (graph of 10), two kernels / this one:
 // OLMoE 32 tokens 7.0 / 6.2, 128 12.3 / 8.1, 1 5.4 / 6.0; Mixtral 1 6.4 / 4.6, 64 7.5 / 6.0, 300
-// 20.3 / 13.5; the fp32 toy layer 64 5.8 / 4.7, 1999 19.9 / 12.0.
+// 20.3 / 13.5; the fp32 toy layer 64 5.8 / 4.7.
 constexpr int kFusedSlice = 512;
 constexpr int kFusedMaxSlices = 8;  // portable cluster size
 // Warps that compute scores: 16 take the 64 experts of one token in one round.
@@ -827,6 +827,9 @@ template <int EPL>
 constexpr int kFusedWarps = EPL == 1 ? 8 : 16;
 template <int EPL>
 constexpr int kFusedThreads = 32 * (kFusedWarps<EPL> + 1);
+// CTAs an SM holds at least: by the register bound up to 32 experts, else one of 17 warps.
+template <int EPL>
+constexpr int kFusedPerSm = EPL == 1 ? 3 : 1;
 template <int EPL, int TT>
 constexpr int kFusedPairs = EPL == 1 && TT == 1 ? 1 : 4;  // Q
 
@@ -845,7 +848,7 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 template <typename TX, int EPL, int TT>
-__global__ void __launch_bounds__(kFusedThreads<EPL>, EPL == 1 ? 3 : 1)
+__global__ void __launch_bounds__(kFusedThreads<EPL>, kFusedPerSm<EPL>)
 route_fused_kernel(const TX* __restrict__ x, const float* __restrict__ wr, int d, const SelectArgs a,
                    TX* __restrict__ xcopy) {
   using X4 = decltype(load_x4((const TX*)nullptr));
@@ -1064,12 +1067,27 @@ static bool router_vec_ok(const void* x, const float* w_router, int d) {
 }
 
 // One launch for scores and selection: every call of up to kSmallT tokens (d up to 4096, a cluster
-// of at most eight slices), and larger ones of fp32 x or few experts, where the tiled kernels'
-// 64-expert tiles would be mostly empty (Mixtral's 8 experts, us per routing call tiled / fused: 300
-// tokens 20.3 / 13.5, 500 20.7 / 19.7, 1000 28.6 / 42; OLMoE's 64: 200 tokens 14.4 / 16.8).
+// of at most eight slices), and some larger ones (us per routing call, tiled / fused):
+//   bf16 x: few experts, where the tiled kernels' 64-expert tiles would be mostly empty.  Mixtral's 8
+//     experts: 300 tokens 20.3 / 13.5, 500 20.7 / 19.7, 1000 28.6 / 42; OLMoE's 64: 200 14.4 / 16.8.
+//   fp32 x, up to 128 experts: while the clusters of four tokens run in one wave.  64 experts, d 256:
+//     512 tokens 12.3 / 8.6, 768 12.4 / 16.1; d 1024: 300 15.0 / 9.1, 400 15.0 / 16.9; d 2048: 129 16.0
+//     / 9.1, 200 16.0 / 17.1, 4096 57 / 240; 128 experts, d 1024: 300 16.6 / 13.6, 400 19.5 / 25.5; 8
+//     experts, d 256: 1536 11.3 / 7.6, 2048 11.5 / 12.0.  256 experts gain in some waves and lose in
+//     others: d 256: 200 16.3 / 21.8; d 1024: 129 20.3 / 23.0, 300 25.8 / 23.6.
+//   fp32 x, up to 16 experts: also beyond one wave, where W_r read again for every four tokens stays
+//     below 3 * 2^23 products in all.  8 experts, d 1024: 3000 26.7 / 26.1; d 2048: 1536 31.2 / 27.5,
+//     2048 32.9 / 34.7; d 4096: 768 32.5 / 28.4, 1536 48.3 / 54.9; 16 experts, d 512: 3000 19.8 / 16.9,
+//     4096 18.8 / 22.7; d 2048: 768 22.8 / 17.4, 1000 25.1 / 24.1, 1536 31.2 / 32.8.
 bool route_fused(const void* x, int x_bf16, const float* w_router, int T, int d, int E) {
-  return router_vec_ok(x, w_router, d) && d <= kFusedSlice * kFusedMaxSlices &&
-         (T <= kSmallT || !x_bf16 || (long long)T * E <= 4096);
+  if (!router_vec_ok(x, w_router, d) || d > kFusedSlice * kFusedMaxSlices) return false;
+  if (T <= kSmallT) return true;
+  if (x_bf16) return (long long)T * E <= 4096;
+  int sms = 0, per_sm = 0;
+  if (!sk_device(sms, per_sm)) return false;
+  const long long ctas = (long long)((T + 3) / 4) * ((d + kFusedSlice - 1) / kFusedSlice);
+  if (E <= 128 && ctas <= (long long)sms * (E <= 32 ? kFusedPerSm<1> : kFusedPerSm<2>)) return true;
+  return E <= 16 && d >= 512 && T <= 3072 && (long long)T * E * d <= 3LL << 23;
 }
 
 bool router_copies_x(const void* x, int x_bf16, const float* w_router, int T, int d, int E) {

@@ -337,6 +337,37 @@ def test_small_call_routing(dtype, E, d, Ts):
     L.close()
 
 
+@pytest.mark.parametrize("E,d,calls", [
+    # (tokens, in one launch); n: the GPU's SMs
+    (64, 512, lambda n: [(4 * n, True), (4 * n + 1, False)]),     # a CTA per SM, four tokens each
+    (100, 1024, lambda n: [(2 * n, True), (2 * n + 1, False), (4096, False)]),  # two slices
+    (8, 256, lambda n: [(12 * n, True), (12 * n + 1, False)]),    # three CTAs per SM
+    (16, 2048, lambda n: [(768, True), (769, False)]),            # 3 * 2^23 products
+    (256, 256, lambda n: [(129, False), (300, False)]),           # more than 128 experts
+])
+def test_fp32_routing_in_one_launch_up_to_its_line(E, d, calls):
+    """fp32 hidden states above 128 tokens: scores and selection share a launch up to the size where
+    the tiled kernels are faster, and both sides of the line agree with the oracle."""
+    cases = calls(torch.cuda.get_device_properties(0).multi_processor_count)
+    sh = W.scaled(W.OLMOE, f"fl{E}-{d}", d_model=d, n_experts=E, d_ff=64, max_k=min(E, 5),
+                  wdtype=torch.float32, xdtype=torch.float32)
+    lw = W.make_layer(sh)
+    ref = oracle_layer(lw)
+    L = eat.EatLayer.from_workload(lw, max(T for T, _ in cases), gpu_params(sh))
+    L.forward(W.make_tokens(sh, 50, step=9).cuda(), 0)
+    acc = _acc(L)
+    prm = orc.Params(max_k=sh.max_k, temperature=sh.temperature)
+    for T, one in cases:
+        x = W.make_tokens(sh, T, step=T).cuda()
+        eat.eat_profile_begin(L.h, 4)
+        idx, w, k = L.route(x, 0)
+        prof = eat.eat_profile_end(L.h)
+        assert (prof["route"][1], prof["select"][1]) == ((1, 0) if one else (1, 1)), T
+        routing = orc.route(np64(x), ref, acc, prm, 0)
+        par.check_routing(routing, par.gpu_selection(idx, k), w.cpu().numpy(), sh.max_k)
+    L.close()
+
+
 @pytest.mark.parametrize("which", ["all", "some", "misaligned"])
 def test_routing_and_account_outputs(which):
     """The caller's routing buffers, all, some or (misaligned) copied at the end, hold what eat_route
