@@ -199,8 +199,9 @@ eat_status check_call(eat_handle* h, const void* x, int32_t T, int32_t ppl_sign)
   return check_state(h);
 }
 
-// Router + selection into (idx, w, k, psel), and into the caller's copies.  x_host (or null): the router kernel reads the
-// tokens there (a page-locked host buffer) and writes them to x, which later kernels read.
+// Router + selection into (idx, w, k, psel), and into the caller's copies.  x_host (or null): the
+// router kernel reads the tokens there (a page-locked host buffer) and writes them to x, which later
+// kernels read.
 eat_status run_route(eat_handle* h, const void* x, int T, int ppl_sign, int32_t* idx, float* w,
                      int32_t* k, float* psel, RouteCopies copies, bool write_tau, cudaStream_t st,
                      const void* x_host = nullptr) {

@@ -1398,94 +1398,99 @@ template <int BN, int MODE, bool W8, bool TOK>
 cudaError_t launch_tc(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
                       const TcArgs& args, int grid, cudaStream_t st) {
   using C = Cfg<BN, MODE, W8>;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  std::call_once(once, [] {
-    attr_err = cudaFuncSetAttribute(tc_ffn_kernel<BN, MODE, W8, TOK>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-  });
-  if (attr_err != cudaSuccess) return attr_err;
   if (grid <= 0) return cudaSuccess;
   return launch_pdl(tc_ffn_kernel<BN, MODE, W8, TOK>, dim3(grid), dim3(C::kThreads), C::kSmemBytes,
                     st, a0, a1, b, args);
+}
+// Lets the kernel use its shared memory in the current context (tc_configure, per handle).
+template <int BN, int MODE, bool W8, bool TOK>
+cudaError_t configure_tc() {
+  return cudaFuncSetAttribute(tc_ffn_kernel<BN, MODE, W8, TOK>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              Cfg<BN, MODE, W8>::kSmemBytes);
 }
 
 // SM-pair kernels: one 2-CTA cluster per pair of SMs, at most as many pairs as can be resident.
 // The routed set (a0, a1, b, args) and, when sargs is given, the shared set of the same call in
 // the same launch; units counts both.
+template <int MODE, bool FOLD, bool IL4, int KPS>
+constexpr int kPairId = (MODE == kModeDown ? 0 : 1) + 2 * FOLD + 4 * IL4 + 8 * (KPS == 1);
+static_assert(kPairId<kModeGateUpIL, true, true, 1> < TcLayer::kPairKernels, "max_pairs entries");
 template <int MODE, bool FOLD, bool IL4, bool W8 = false, int KPS = 2>
-cudaError_t launch_pair_t(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
-                          const TcArgs& args, long long units, int num_sms, cudaStream_t st,
-                          const CUtensorMap* sa0, const CUtensorMap* sa1, const CUtensorMap* sb,
-                          const TcArgs* sargs) {
+cudaError_t launch_pair_t(const TcLayer& L, const CUtensorMap& a0, const CUtensorMap& a1,
+                          const CUtensorMap& b, const TcArgs& args, long long units,
+                          cudaStream_t st, const CUtensorMap* sa0, const CUtensorMap* sa1,
+                          const CUtensorMap* sb, const TcArgs* sargs) {
   using C = PairCfg<MODE, IL4, W8, KPS>;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  static int max_pairs = 0;
-  std::call_once(once, [num_sms] {
-    attr_err = cudaFuncSetAttribute(tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-    if (attr_err != cudaSuccess) return;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(num_sms & ~1);
-    cfg.blockDim = dim3(C::kThreads);
-    cfg.dynamicSmemBytes = C::kSmemBytes;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>, &cfg) != cudaSuccess ||
-        n <= 0) {
-      cudaGetLastError();
-      n = num_sms / 2;
-    }
-    max_pairs = std::min(n, num_sms / 2);
-  });
-  if (attr_err != cudaSuccess) return attr_err;
-  const long long pairs = std::min<long long>(max_pairs, units);
-  if (pairs <= 0) return cudaSuccess;
+  const long long pairs =
+      std::min<long long>(L.max_pairs[kPairId<MODE, FOLD, IL4, KPS>], units);
+  if (pairs <= 0) return units <= 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
   TcArgs none;
   std::memset(&none, 0, sizeof(none));
   return launch_pdl(tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>, dim3((unsigned)(2 * pairs)), dim3(C::kThreads),
                     C::kSmemBytes, st, a0, a1, b, args, sa0 ? *sa0 : a0, sa1 ? *sa1 : a1,
                     sb ? *sb : b, sargs ? *sargs : none);
 }
+// The same for an SM-pair kernel, and the number of its clusters that can be resident.
+template <int MODE, bool FOLD, bool IL4, bool W8 = false, int KPS = 2>
+cudaError_t configure_pair(TcLayer& L) {
+  using C = PairCfg<MODE, IL4, W8, KPS>;
+  const cudaError_t e =
+      cudaFuncSetAttribute(tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(L.num_sms & ~1);
+  cfg.blockDim = dim3(C::kThreads);
+  cfg.dynamicSmemBytes = C::kSmemBytes;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, tc_pair_kernel<MODE, FOLD, IL4, W8, KPS>, &cfg) !=
+          cudaSuccess ||
+      n <= 0) {
+    cudaGetLastError();
+    n = L.num_sms / 2;
+  }
+  L.max_pairs[kPairId<MODE, FOLD, IL4, KPS>] = std::min(n, L.num_sms / 2);
+  return cudaSuccess;
+}
 // KPS: k-blocks per pipeline stage (one only for the 16-row interleaved gate/up and the down
 // projection, whose shared memory holds seven stages).
 template <int MODE, bool IL4, int KPS>
-cudaError_t launch_pair_k(const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
-                          const TcArgs& args, long long units, int num_sms, cudaStream_t st,
-                          const CUtensorMap* sa0, const CUtensorMap* sa1, const CUtensorMap* sb,
-                          const TcArgs* sargs) {
+cudaError_t launch_pair_k(const TcLayer& L, const CUtensorMap& a0, const CUtensorMap& a1,
+                          const CUtensorMap& b, const TcArgs& args, long long units,
+                          cudaStream_t st, const CUtensorMap* sa0, const CUtensorMap* sa1,
+                          const CUtensorMap* sb, const TcArgs* sargs) {
   if (sargs)
-    return launch_pair_t<MODE, true, IL4, false, KPS>(a0, a1, b, args, units, num_sms, st, sa0, sa1,
-                                                      sb, sargs);
-  return launch_pair_t<MODE, false, IL4, false, KPS>(a0, a1, b, args, units, num_sms, st, nullptr,
-                                                     nullptr, nullptr, nullptr);
+    return launch_pair_t<MODE, true, IL4, false, KPS>(L, a0, a1, b, args, units, st, sa0, sa1, sb,
+                                                      sargs);
+  return launch_pair_t<MODE, false, IL4, false, KPS>(L, a0, a1, b, args, units, st, nullptr, nullptr,
+                                                     nullptr, nullptr);
 }
 template <int MODE, bool IL4 = false>
-cudaError_t launch_pair(bool one_kb, const CUtensorMap& a0, const CUtensorMap& a1,
-                        const CUtensorMap& b, const TcArgs& args, long long units, int num_sms,
-                        cudaStream_t st, const CUtensorMap* sa0 = nullptr,
-                        const CUtensorMap* sa1 = nullptr, const CUtensorMap* sb = nullptr,
-                        const TcArgs* sargs = nullptr) {
+cudaError_t launch_pair(const TcLayer& L, bool one_kb, const CUtensorMap& a0, const CUtensorMap& a1,
+                        const CUtensorMap& b, const TcArgs& args, long long units, cudaStream_t st,
+                        const CUtensorMap* sa0 = nullptr, const CUtensorMap* sa1 = nullptr,
+                        const CUtensorMap* sb = nullptr, const TcArgs* sargs = nullptr) {
   if constexpr (IL4 || MODE == kModeDown) {
     if (one_kb)
-      return launch_pair_k<MODE, IL4, 1>(a0, a1, b, args, units, num_sms, st, sa0, sa1, sb, sargs);
+      return launch_pair_k<MODE, IL4, 1>(L, a0, a1, b, args, units, st, sa0, sa1, sb, sargs);
   }
-  return launch_pair_k<MODE, IL4, 2>(a0, a1, b, args, units, num_sms, st, sa0, sa1, sb, sargs);
+  return launch_pair_k<MODE, IL4, 2>(L, a0, a1, b, args, units, st, sa0, sa1, sb, sargs);
 }
 
 // fp8: one unit set (the gate/up map is the 16-row interleaved view).
 template <int MODE>
-cudaError_t launch_pair8(const CUtensorMap& a, const CUtensorMap& b, const TcArgs& args,
-                         long long units, int num_sms, cudaStream_t st) {
-  return launch_pair_t<MODE, false, MODE == kModeGateUpIL, true>(a, a, b, args, units, num_sms, st,
-                                                                 nullptr, nullptr, nullptr, nullptr);
+cudaError_t launch_pair8(const TcLayer& L, const CUtensorMap& a, const CUtensorMap& b,
+                         const TcArgs& args, long long units, cudaStream_t st) {
+  return launch_pair_t<MODE, false, MODE == kModeGateUpIL, true>(L, a, a, b, args, units, st, nullptr,
+                                                                 nullptr, nullptr, nullptr);
 }
 
 // Single-SM launches: token tiles of 16..128 rows (256-row tiles run on SM pairs); W8 for fp8
@@ -1499,6 +1504,46 @@ cudaError_t launch_bn(int bn, const CUtensorMap& a0, const CUtensorMap& a1, cons
     case 64: return launch_tc<64, MODE, W8, TOK>(a0, a1, b, args, grid, st);
     default: return launch_tc<128, MODE, W8, TOK>(a0, a1, b, args, grid, st);
   }
+}
+
+template <int MODE, bool W8, bool TOK>
+cudaError_t configure_bn() {
+  cudaError_t e = configure_tc<16, MODE, W8, TOK>();
+  if (e == cudaSuccess) e = configure_tc<32, MODE, W8, TOK>();
+  if (e == cudaSuccess) e = configure_tc<64, MODE, W8, TOK>();
+  if (e == cudaSuccess) e = configure_tc<128, MODE, W8, TOK>();
+  return e;
+}
+template <int MODE, bool IL4>
+cudaError_t configure_pairs(TcLayer& L) {
+  cudaError_t e = configure_pair<MODE, false, IL4>(L);
+  if (e == cudaSuccess && L.S > 0) e = configure_pair<MODE, true, IL4>(L);
+  if constexpr (IL4 || MODE == kModeDown) {
+    if (e == cudaSuccess) e = configure_pair<MODE, false, IL4, false, 1>(L);
+    if (e == cudaSuccess && L.S > 0) e = configure_pair<MODE, true, IL4, false, 1>(L);
+  }
+  return e;
+}
+// Every kernel that a handle of this type may launch (the attributes hold for the current context
+// only, so this runs for each handle and not once per process).
+cudaError_t configure_kernels(TcLayer& L) {
+  const bool pairs = L.Tmax > kBNs[kNumBN - 1];
+  cudaError_t e;
+  if (L.w8) {
+    e = configure_bn<kModeGateUp, true, false>();
+    if (e == cudaSuccess) e = configure_bn<kModeDown, true, false>();
+    if (e == cudaSuccess && pairs) e = configure_pair<kModeGateUpIL, false, true, true>(L);
+    if (e == cudaSuccess && pairs) e = configure_pair<kModeDown, false, false, true>(L);
+    return e;
+  }
+  e = configure_bn<kModeGateUp, false, false>();
+  if (e == cudaSuccess) e = configure_bn<kModeGateUp, false, true>();
+  if (e == cudaSuccess) e = configure_bn<kModeGateUpIL, false, true>();
+  if (e == cudaSuccess) e = configure_bn<kModeDown, false, false>();
+  if (e == cudaSuccess && pairs) e = configure_pairs<kModeGateUpIL, true>(L);
+  if (e == cudaSuccess && pairs) e = configure_pairs<kModeGateUpIL, false>(L);
+  if (e == cudaSuccess && pairs) e = configure_pairs<kModeDown, false>(L);
+  return e;
 }
 
 }  // namespace
@@ -1632,6 +1677,11 @@ int tc_configure(TcLayer& L, const eat_layer_desc& D, int K, int Tmax, const cha
     return 1;
   }
   L.num_sms = prop.multiProcessorCount;
+  const cudaError_t e = configure_kernels(L);
+  if (e != cudaSuccess) {
+    if (msg) *msg = cudaGetErrorString(e);
+    return 1;
+  }
   if (!encode_fn()) {
     if (msg) *msg = "cuTensorMapEncodeTiled is unavailable";
     return 1;
@@ -1772,18 +1822,16 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     if (shared) {
       shared_args(a);
       a.gate_first = m->sgate_first ? 1 : 0;
-      return launch_pair8<kModeGateUpIL>(m->wsgu4, m->xqt[bn_index(kPairRows / 2)], a,
-                                         (long long)L.S * ((c.T + bn - 1) / bn) * a.m_tiles,
-                                         L.num_sms, st);
+      return launch_pair8<kModeGateUpIL>(L, m->wsgu4, m->xqt[bn_index(kPairRows / 2)], a,
+                                         (long long)L.S * ((c.T + bn - 1) / bn) * a.m_tiles, st);
     }
     a.gate_first = m->gate_first ? 1 : 0;
     a.n_groups = L.E;
     a.row_offs = c.offs;
     a.tile_offs = c.tile_offs;
     a.out = c.act;
-    return launch_pair8<kModeGateUpIL>(m->wgu4, m->xq[bn_index(kPairRows / 2)], a,
-                                       ((long long)(c.T * L.K + bn - 1) / bn + L.E) * a.m_tiles,
-                                       L.num_sms, st);
+    return launch_pair8<kModeGateUpIL>(L, m->wgu4, m->xq[bn_index(kPairRows / 2)], a,
+                                       ((long long)(c.T * L.K + bn - 1) / bn + L.E) * a.m_tiles, st);
   }
   if (shared) {
     CUtensorMap xm;
@@ -1794,11 +1842,10 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     const long long units = max_tiles * a.m_tiles;
     if (pair && m->sil4) {
       a.gate_first = m->sgate_first ? 1 : 0;
-      return launch_pair<kModeGateUpIL, true>(one_kb, m->wsgu4, m->wsgu4, xm, a, units, L.num_sms,
-                                              st);
+      return launch_pair<kModeGateUpIL, true>(L, one_kb, m->wsgu4, m->wsgu4, xm, a, units, st);
     }
     if (pair)
-      return launch_pair<kModeGateUpIL>(one_kb, m->wsg64, m->wsu64, xm, a, units, L.num_sms, st);
+      return launch_pair<kModeGateUpIL>(L, one_kb, m->wsg64, m->wsu64, xm, a, units, st);
     const int grid = (int)std::min<long long>(L.num_sms, units);
     return up_bn(m->wsg, m->wsu, xm, grid);
   }
@@ -1836,22 +1883,21 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     if (m->il4 && m->sil4) {
       a.gate_first = m->gate_first ? 1 : 0;
       sa.gate_first = m->sgate_first ? 1 : 0;
-      return launch_pair<kModeGateUpIL, true>(one_kb, m->wgu4, m->wgu4,
+      return launch_pair<kModeGateUpIL, true>(L, one_kb, m->wgu4, m->wgu4,
                                               m->xperm[bn_index(kPairRows)], a, units + s_units,
-                                              L.num_sms, st, &m->wsgu4, &m->wsgu4, &xm, &sa);
+                                              st, &m->wsgu4, &m->wsgu4, &xm, &sa);
     }
-    return launch_pair<kModeGateUpIL>(one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
-                                      units + s_units, L.num_sms, st, &m->wsg64, &m->wsu64, &xm,
-                                      &sa);
+    return launch_pair<kModeGateUpIL>(L, one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
+                                      units + s_units, st, &m->wsg64, &m->wsu64, &xm, &sa);
   }
   if (pair && m->il4) {
     a.gate_first = m->gate_first ? 1 : 0;
-    return launch_pair<kModeGateUpIL, true>(one_kb, m->wgu4, m->wgu4,
-                                            m->xperm[bn_index(kPairRows)], a, units, L.num_sms, st);
+    return launch_pair<kModeGateUpIL, true>(L, one_kb, m->wgu4, m->wgu4,
+                                            m->xperm[bn_index(kPairRows)], a, units, st);
   }
   if (pair)
-    return launch_pair<kModeGateUpIL>(one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
-                                      units, L.num_sms, st);
+    return launch_pair<kModeGateUpIL>(L, one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
+                                      units, st);
   return up_bn(m->wg, m->wu, L.w8 ? m->xq[bn_index(bn)] : m->xperm[bn_index(bn)], grid);
 }
 
@@ -1910,10 +1956,10 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
     max_tiles = (long long)L.S * ((c.T + bn - 1) / bn);
     const long long units = max_tiles * a.m_tiles;
     if (pair8)
-      return launch_pair8<kModeDown>(m->wsd, m->saq[bn_index(kPairRows)], a, units, L.num_sms, st);
+      return launch_pair8<kModeDown>(L, m->wsd, m->saq[bn_index(kPairRows)], a, units, st);
     if (pair)
-      return launch_pair<kModeDown>(one_kb, m->wsd, m->wsd, m->sact[bn_index(kPairRows)], a, units,
-                                    L.num_sms, st);
+      return launch_pair<kModeDown>(L, one_kb, m->wsd, m->wsd, m->sact[bn_index(kPairRows)], a,
+                                    units, st);
     const int grid = (int)std::min<long long>(L.num_sms, units);
     return down_bn(m->wsd, L.w8 ? m->saq[bn_index(bn)] : m->sact[bn_index(bn)], grid);
   }
@@ -1929,16 +1975,14 @@ cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n
     TcArgs sa;
     shared_args(sa);
     const long long s_units = (long long)L.S * ((c.T + bn - 1) / bn) * sa.m_tiles;
-    return launch_pair<kModeDown>(one_kb, m->wd, m->wd, m->act[bn_index(kPairRows)], a,
-                                  units + s_units,
-                                  L.num_sms, st, &m->wsd, &m->wsd,
+    return launch_pair<kModeDown>(L, one_kb, m->wd, m->wd, m->act[bn_index(kPairRows)], a,
+                                  units + s_units, st, &m->wsd, &m->wsd,
                                   &m->sact[bn_index(kPairRows)], &sa);
   }
   if (pair8)
-    return launch_pair8<kModeDown>(m->wd, m->aq[bn_index(kPairRows)], a, units, L.num_sms, st);
+    return launch_pair8<kModeDown>(L, m->wd, m->aq[bn_index(kPairRows)], a, units, st);
   if (pair)
-    return launch_pair<kModeDown>(one_kb, m->wd, m->wd, m->act[bn_index(kPairRows)], a, units,
-                                  L.num_sms,
+    return launch_pair<kModeDown>(L, one_kb, m->wd, m->wd, m->act[bn_index(kPairRows)], a, units,
                                   st);
   const int grid = (int)std::min<long long>(L.num_sms, units);
   return down_bn(m->wd, L.w8 ? m->aq[bn_index(bn)] : m->act[bn_index(bn)], grid);

@@ -23,6 +23,9 @@ struct TcLayer {
   bool ready = false;
   int E = 0, d = 0, F = 0, S = 0, Fs = 0, K = 0, Tmax = 0;
   int num_sms = 0;
+  // SM-pair clusters that can be resident, per kernel (kPairId in ffn_tc.cu)
+  static constexpr int kPairKernels = 16;
+  int max_pairs[kPairKernels] = {};
   bool w8 = false;  // e4m3 expert weights with per-row fp32 scales (kind::f8f6f4 MMAs)
   const float *sg = nullptr, *su = nullptr, *sd = nullptr;     // [E,F], [E,F], [E,d]
   const float *ssg = nullptr, *ssu = nullptr, *ssd = nullptr;  // shared experts
