@@ -216,8 +216,8 @@ eat_status eat_moe_forward_host_async(eat_handle* h, const void* x_host, int32_t
  * the library, which every GPU that loads the library holds until the process exits.
  *  - T * n_experts must be <= 131072 (EAT_NOALLOC_SCRATCH_BYTES / 8), else EAT_ERR_INVALID_ARG;
  *    larger batches are routed in several calls.
- *  - The first call on each device looks up the scratch's device address (a one-time set-up per
- *    device, done with that device current), and so does the first call after the device's
+ *  - The first call on each device looks up the scratch's device address and sets the router
+ *    kernels up (once per device, with that device current), and so does the first call after the device's
  *    current context changed (e.g. after cudaDeviceReset); make that first call before any
  *    stream capture.
  *  - Calls share the scratch: two calls that may overlap on the GPU (different streams or host

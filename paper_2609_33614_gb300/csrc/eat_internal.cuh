@@ -20,6 +20,10 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 
 bool pdl_enabled();
 
+// Unique id of the context current on this thread; false if there is none or the driver cannot tell.
+// (After cudaDeviceReset the device's next context has another one.)
+bool current_context_id(unsigned long long* id);
+
 // Compensated fp32 sums ("double-float": a value is the unevaluated sum hi + lo).  GB300's fp64
 // pipe runs about two lanes per SM per clock, so one fp64 warp instruction occupies it for ~64
 // cycles; sums that need more than fp32 precision use these error-free fp32 steps instead.
@@ -142,6 +146,9 @@ cudaError_t launch_route_select(const float2* part, int n_split, const float* b_
                                 int E, int K, const int64_t* accN, const double* accP,
                                 const double* accC, RouteParams rp, int32_t* idx, float* w,
                                 int32_t* k, float* psel, RouteCopies copies, cudaStream_t st);
+// The routers' one-time set-up in the current context, which the first call that needs it makes
+// otherwise; false without a device.
+bool router_setup();
 constexpr int kRouterTileT = 64;    // tokens of a tile of the larger calls' routers
 constexpr int kSmallRouterT = 128;  // calls up to this many tokens use the GEMV-style router
 int router_split(int T, int d, int E);

@@ -22,12 +22,14 @@
 
 #include <algorithm>
 #include <atomic>
+#include <mutex>
 
 namespace eat {
 
 namespace {
 
 constexpr int kLogitThreads = 256;
+constexpr int kMaxRouterDevices = 64;
 
 __device__ __forceinline__ float load_x(const float* p, size_t i) { return p[i]; }
 __device__ __forceinline__ float load_x(const __nv_bfloat16* p, size_t i) {
@@ -978,19 +980,23 @@ route_fused_kernel(const TX* __restrict__ x, const float* __restrict__ wr, int d
 
 namespace {
 
-// CTAs of router_logits_sk_kernel resident per SM, and the SM count, of the current device (both
-// queried once per device; concurrent first calls compute the same values)
+// CTAs of router_logits_sk_kernel resident per SM, and the SM count, of the current device, with the
+// kernel's shared-memory limit raised: once per device and context (a reset device has lost the limit)
 struct SkDevice {
-  std::atomic<int> ready{0};
-  int sms = 0, per_sm = 0;
+  unsigned long long ctx_id = 0;
+  int sms = 0, per_sm = 0;  // 0: not set up
 };
-SkDevice g_sk_dev[64];
+std::mutex g_sk_mu;
+SkDevice g_sk_dev[kMaxRouterDevices];
 
 bool sk_device(int& sms, int& per_sm) {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxRouterDevices) return false;
+  std::lock_guard<std::mutex> lock(g_sk_mu);
   SkDevice& D = g_sk_dev[dev];
-  if (!D.ready.load(std::memory_order_acquire)) {
+  unsigned long long id = 0;
+  if (!(D.sms && current_context_id(&id) && id == D.ctx_id)) {
+    D = {};
     int n = 0, b = 0;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaFuncSetAttribute(router_logits_sk_kernel<kSKTM>,
@@ -999,12 +1005,28 @@ bool sk_device(int& sms, int& per_sm) {
                                                       SkCfg<kSKTM>::kThreads, kSKSmem) != cudaSuccess ||
         n < 1 || b < 1)
       return false;
-    D.sms = n;
-    D.per_sm = b;
-    D.ready.store(1, std::memory_order_release);
+    sms = n;
+    per_sm = b;
+    // (the set-up made the device's primary context current if none was; a context that the driver
+    // cannot identify is set up by every call)
+    if (current_context_id(&id)) D = {id, n, b};
+    return true;
   }
   sms = D.sms;
   per_sm = D.per_sm;
+  return true;
+}
+
+// The SM count alone, which outlives contexts: what the one-launch router needs.
+bool device_sms(int& sms) {
+  static std::atomic<int> cached[kMaxRouterDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxRouterDevices) return false;
+  sms = cached[dev].load(std::memory_order_relaxed);
+  if (sms > 0) return true;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return false;
+  cached[dev].store(sms, std::memory_order_relaxed);
   return true;
 }
 
@@ -1046,6 +1068,11 @@ bool sk_eligible(int T, int d) { return T > kSmallT && d % kChunkK == 0; }
 
 }  // namespace
 
+bool router_setup() {
+  int sms = 0, per_sm = 0;
+  return sk_device(sms, per_sm);
+}
+
 // (eat_create relies on the split of a call being the same for all T with the same number of
 // kRouterTileT-token tiles, up to kSmallRouterT and beyond it)
 static_assert(kSmallT % kRouterTileT == 0, "the small calls end at a tile");
@@ -1083,8 +1110,8 @@ bool route_fused(const void* x, int x_bf16, const float* w_router, int T, int d,
   if (!router_vec_ok(x, w_router, d) || d > kFusedSlice * kFusedMaxSlices) return false;
   if (T <= kSmallT) return true;
   if (x_bf16) return (long long)T * E <= 4096;
-  int sms = 0, per_sm = 0;
-  if (!sk_device(sms, per_sm)) return false;
+  int sms = 0;
+  if (!device_sms(sms)) return false;
   const long long ctas = (long long)((T + 3) / 4) * ((d + kFusedSlice - 1) / kFusedSlice);
   if (E <= 128 && ctas <= (long long)sms * (E <= 32 ? kFusedPerSm<1> : kFusedPerSm<2>)) return true;
   return E <= 16 && d >= 512 && T <= 3072 && (long long)T * E * d <= 3LL << 23;
@@ -1158,8 +1185,8 @@ namespace {
 template <typename TX, int EPL>
 cudaError_t launch_fused_t(const TX* x, const float* wr, int d, const SelectArgs& a, TX* xcopy,
                            cudaStream_t st) {
-  int sms = 0, per_sm = 0;
-  if (!sk_device(sms, per_sm)) return cudaErrorInvalidDevice;
+  int sms = 0;
+  if (!device_sms(sms)) return cudaErrorInvalidDevice;
   const int nsl = (d + kFusedSlice - 1) / kFusedSlice;
   if (a.T * nsl <= sms)
     return launch_pdl_cluster(route_fused_kernel<TX, EPL, 1>, dim3(nsl, a.T), nsl,

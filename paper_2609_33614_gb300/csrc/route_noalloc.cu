@@ -36,9 +36,57 @@ struct Cached {
 };
 Cached g_scratch[kMaxDevices];
 
-// Unique id of the context current on this thread (driver entry points fetched through the
-// runtime, so the library needs no link against the driver library); false if there is none or
-// the driver cannot tell.
+// Device address of the scratch in the current device's current context.  In host code
+// g_route_scratch names a host-side stand-in, not device memory, so only this address may be
+// handed to a kernel.  It is looked up once per device, with that device current, and again
+// whenever the device's current context is another one than at the last look-up (after
+// cudaDeviceReset the module is loaded anew and the array may move).
+eat_status scratch_address(float2** out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) {
+    eat::set_thread_error((std::string("cudaGetDevice: ") + cudaGetErrorString(e)).c_str());
+    return EAT_ERR_CUDA;
+  }
+  if (dev < 0 || dev >= kMaxDevices) {
+    eat::set_thread_error("device index beyond the 64 devices eat_route_noalloc supports");
+    return EAT_ERR_UNSUPPORTED;
+  }
+  std::lock_guard<std::mutex> lock(g_mu);
+  unsigned long long id = 0;
+  if (g_scratch[dev].ptr && eat::current_context_id(&id) && id == g_scratch[dev].ctx_id) {
+    *out = (float2*)g_scratch[dev].ptr;
+    return EAT_OK;
+  }
+  if (!eat::router_setup()) {  // (the kernels' set-up in this context, also for larger calls)
+    eat::set_thread_error("eat_route_noalloc: the router kernels cannot be set up on this device");
+    return EAT_ERR_CUDA;
+  }
+  void* p = nullptr;
+  e = cudaGetSymbolAddress(&p, g_route_scratch);
+  if (e != cudaSuccess || !p) {
+    eat::set_thread_error((std::string("cudaGetSymbolAddress of the routing scratch: ") +
+                           cudaGetErrorString(e)).c_str());
+    return EAT_ERR_CUDA;
+  }
+  // the look-up made the device's primary context current if none was; a context the driver
+  // cannot identify is not cached (then every call looks the address up)
+  if (eat::current_context_id(&id)) g_scratch[dev] = {id, p};
+  else g_scratch[dev] = {};
+  *out = (float2*)p;
+  return EAT_OK;
+}
+
+eat_status bad(const char* msg) {
+  eat::set_thread_error(msg);
+  return EAT_ERR_INVALID_ARG;
+}
+
+}  // namespace
+
+namespace eat {
+// (driver entry points fetched through the runtime, so the library needs no link against the driver
+// library)
 bool current_context_id(unsigned long long* id) {
   static PFN_cuCtxGetCurrent_v4000 get_cur = nullptr;
   static PFN_cuCtxGetId_v12000 get_id = nullptr;
@@ -58,50 +106,7 @@ bool current_context_id(unsigned long long* id) {
   if (!get_cur || !get_id || get_cur(&c) != CUDA_SUCCESS || !c) return false;
   return get_id(c, id) == CUDA_SUCCESS;
 }
-
-// Device address of the scratch in the current device's current context.  In host code
-// g_route_scratch names a host-side stand-in, not device memory, so only this address may be
-// handed to a kernel.  It is looked up once per device, with that device current, and again
-// whenever the device's current context is another one than at the last look-up (after
-// cudaDeviceReset the module is loaded anew and the array may move).
-eat_status scratch_address(float2** out) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) {
-    eat::set_thread_error((std::string("cudaGetDevice: ") + cudaGetErrorString(e)).c_str());
-    return EAT_ERR_CUDA;
-  }
-  if (dev < 0 || dev >= kMaxDevices) {
-    eat::set_thread_error("device index beyond the 64 devices eat_route_noalloc supports");
-    return EAT_ERR_UNSUPPORTED;
-  }
-  std::lock_guard<std::mutex> lock(g_mu);
-  unsigned long long id = 0;
-  if (g_scratch[dev].ptr && current_context_id(&id) && id == g_scratch[dev].ctx_id) {
-    *out = (float2*)g_scratch[dev].ptr;
-    return EAT_OK;
-  }
-  void* p = nullptr;
-  e = cudaGetSymbolAddress(&p, g_route_scratch);
-  if (e != cudaSuccess || !p) {
-    eat::set_thread_error((std::string("cudaGetSymbolAddress of the routing scratch: ") +
-                           cudaGetErrorString(e)).c_str());
-    return EAT_ERR_CUDA;
-  }
-  // the look-up made the device's primary context current if none was; a context the driver
-  // cannot identify is not cached (then every call looks the address up)
-  if (current_context_id(&id)) g_scratch[dev] = {id, p};
-  else g_scratch[dev] = {};
-  *out = (float2*)p;
-  return EAT_OK;
-}
-
-eat_status bad(const char* msg) {
-  eat::set_thread_error(msg);
-  return EAT_ERR_INVALID_ARG;
-}
-
-}  // namespace
+}  // namespace eat
 
 extern "C" eat_status eat_route_noalloc(const void* x, int32_t T, int32_t d_model,
                                         int32_t n_experts, int32_t xdtype, const float* w_router,

@@ -78,3 +78,25 @@ def test_handles_on_two_devices(lib, wdt, xdt):
         lib.fake_set_device(dev)
         for view in (True, False):
             assert _layer_calls(lib, wdt, xdt, Ts, view) == 0  # nothing is left to a handle's calls
+
+
+def _route_noalloc(lib, T):
+    p = eat.eat_default_params(4)
+    a = [4096 * i for i in range(1, 9)]
+    return lib.eat_route_noalloc(a[0], T, 2048, 64, eat.EAT_BF16, a[1], None, a[2], a[3], a[4],
+                                 ctypes.byref(p), 0, a[5], a[6], a[7], None)
+
+
+def test_noalloc_set_up_by_the_first_call_of_a_context(lib):
+    """The first eat_route_noalloc call on a device, of any size, leaves no set-up to later ones (a
+    stream capture may follow it), and so does the first one after the device was reset, which takes
+    the kernels' shared-memory limits."""
+    for dev in (0, 1):
+        lib.fake_set_device(dev)
+        for _ in range(2):
+            assert _route_noalloc(lib, 8) == eat.EAT_OK
+            done = lib.fake_setups()
+            for T in (128, 300, 2048, 1):
+                assert _route_noalloc(lib, T) == eat.EAT_OK, lib.eat_last_error(None)
+            assert lib.fake_setups() == done
+            lib.fake_reset_device()
