@@ -308,6 +308,11 @@ def test_router_runs_split_between_blocks(E, d):
     (torch.bfloat16, 8, 4096, (1, 19, 20, 512)),    # clusters of eight; last call past 128 tokens
     (torch.bfloat16, 256, 576, (2, 77)),            # a 64-column second slice, four rounds of experts
     (torch.bfloat16, 1, 64, (5,)),
+    (torch.bfloat16, 64, 1536, (50, 51, 127)),      # clusters of three, five, six and seven
+    (torch.bfloat16, 40, 2560, (30, 31, 126)),
+    (torch.bfloat16, 16, 3072, (25, 26, 129)),
+    (torch.bfloat16, 64, 3584, (21, 22, 125)),
+    (torch.float32, 130, 3584, (2, 23, 99)),
     (torch.bfloat16, 33, 4160, (1, 128)),           # nine slices: the two-kernel path
     (torch.float32, 100, 640, (3, 300)),            # fp32 hidden states beyond 128 tokens
 ])
@@ -482,7 +487,7 @@ def test_account_update_around_the_one_warp_limit(T):
 
 @pytest.mark.parametrize("E,K,T", [(256, 8, 1500), (64, 2, 1100)])
 def test_sm_pair_small_groups(E, K, T):
-    """Calls of >= 1024 tokens run the SM-pair GEMMs; with many experts nearly every group is a
+    """Large calls (SM-pair GEMMs from 512 tokens on); with many experts nearly every group is a
     partial 256-token tile (MMA widths of 32..224, one CTA's half of the tile empty or partial),
     and the all-tokens-one-expert call below makes one group span several full tiles."""
     sh = W.scaled(W.OLMOE, f"pair{E}", d_model=256, n_experts=E, d_ff=384, max_k=K)

@@ -70,6 +70,31 @@ def test_noalloc_matches_route_and_oracle_two_calls(layer, calls):
         par.check_routing(routing, par.gpu_selection(idx, k), w.cpu().numpy(), SHAPE.max_k)
 
 
+@pytest.mark.parametrize("T", [3, 61, 200])
+@pytest.mark.parametrize("d,off", [(4, 0), (516, 0), (515, 0), (640, 8)])
+def test_noalloc_widths_and_alignments(layer, d, off, T):
+    """Widths that no handle takes (multiples of 4: a short slice of the one-launch router; others: the
+    scalar one) and an x that is not 16-byte aligned (off bytes)."""
+    E, K = 12, 3
+    g = torch.Generator().manual_seed(d + T)
+    x = torch.randn(T, d, generator=g).to(torch.bfloat16)
+    wr = torch.randn(E, d, generator=g) * 0.3
+    buf = torch.zeros(T * d + 16, dtype=torch.bfloat16, device="cuda")
+    xd = buf[off // 2:off // 2 + T * d].view(T, d)
+    xd.copy_(x)
+    acc = [torch.zeros(E, dtype=t, device="cuda") for t in (torch.int64, torch.float64, torch.float64)]
+    idx = torch.full((T, K), -7, dtype=torch.int32, device="cuda")
+    w = torch.full((T, K), -7.0, device="cuda")
+    k = torch.full((T,), -7, dtype=torch.int32, device="cuda")
+    eat.eat_route_noalloc(xd, T, d, E, eat.EAT_BF16, wr.cuda(), None, *acc,
+                          eat.eat_default_params(K), 0, idx, w, k)
+    torch.cuda.synchronize()
+    ref = orc.Layer(np64(wr), None, None, None, None, None, None, None)
+    routing = orc.route(np64(x), ref, orc.Accounts(*(a.cpu().numpy() for a in acc)),
+                        orc.Params(max_k=K), 0)
+    par.check_routing(routing, par.gpu_selection(idx, k), w.cpu().numpy(), K)
+
+
 def test_noalloc_small_call_then_captured_larger_call(layer):
     """A program warms up with a decode batch (one launch, no scratch) and then captures a call that
     uses the scratch."""
