@@ -1382,7 +1382,8 @@ struct Maps {
   CUtensorMap wgu4, wsgu4;
   bool il4 = false, sil4 = false;                   // routed / shared view available
   bool gate_first = true, sgate_first = true;       // gate rows first in the view
-  CUtensorMap xperm[kNumBN], act[kNumBN], sact[kNumBN];
+  CUtensorMap xperm;  // 128-row boxes (smaller tiles read x itself)
+  CUtensorMap act[kNumBN], sact[kNumBN];
   // fp8 layers: the e4m3 hi/lo planes of the B operands (slot rows of x, token rows of x, the
   // routed and the shared activations)
   CUtensorMap xq[kNumBN], xqt[kNumBN], aq[kNumBN], saq[kNumBN];
@@ -1493,8 +1494,8 @@ cudaError_t launch_pair8(const TcLayer& L, const CUtensorMap& a, const CUtensorM
                                                                  nullptr, nullptr, nullptr);
 }
 
-// Single-SM launches: token tiles of 16..128 rows (256-row tiles run on SM pairs); W8 for fp8
-// weights (single-SM kernels only, at any call size).
+// Single-SM launches: token tiles of 16..128 rows (256-row tiles run on SM pairs); W8 for fp8 weights
+// (calls of up to 128 tokens, and the gate/up of larger ones whose weights have no 4D view).
 template <int MODE, bool W8, bool TOK>
 cudaError_t launch_bn(int bn, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& b,
                       const TcArgs& args, int grid, cudaStream_t st) {
@@ -1502,7 +1503,9 @@ cudaError_t launch_bn(int bn, const CUtensorMap& a0, const CUtensorMap& a1, cons
     case 16: return launch_tc<16, MODE, W8, TOK>(a0, a1, b, args, grid, st);
     case 32: return launch_tc<32, MODE, W8, TOK>(a0, a1, b, args, grid, st);
     case 64: return launch_tc<64, MODE, W8, TOK>(a0, a1, b, args, grid, st);
-    default: return launch_tc<128, MODE, W8, TOK>(a0, a1, b, args, grid, st);
+    default:
+      if constexpr (MODE == kModeGateUpIL) return cudaErrorInvalidValue;  // (tiles of up to 64 rows)
+      else return launch_tc<128, MODE, W8, TOK>(a0, a1, b, args, grid, st);
   }
 }
 
@@ -1511,7 +1514,9 @@ cudaError_t configure_bn() {
   cudaError_t e = configure_tc<16, MODE, W8, TOK>();
   if (e == cudaSuccess) e = configure_tc<32, MODE, W8, TOK>();
   if (e == cudaSuccess) e = configure_tc<64, MODE, W8, TOK>();
-  if (e == cudaSuccess) e = configure_tc<128, MODE, W8, TOK>();
+  if constexpr (MODE != kModeGateUpIL) {
+    if (e == cudaSuccess) e = configure_tc<128, MODE, W8, TOK>();
+  }
   return e;
 }
 template <int MODE, bool IL4>
@@ -1740,10 +1745,10 @@ int tc_bind(TcLayer& L, const eat_layer_desc& D, void* xperm, void* act, void* s
              encode_2d_u8(&m->saq[i], q.saq, 2LL * L.S * L.Tmax, L.Fs, kBNs[i]);
       continue;
     }
-    ok = encode_2d(&m->xperm[i], xperm, rows, L.d, kBNs[i]) &&
-         encode_2d(&m->act[i], act, rows, L.F, kBNs[i]);
+    ok = encode_2d(&m->act[i], act, rows, L.F, kBNs[i]);
     if (ok && L.S > 0) ok = encode_2d(&m->sact[i], sact, (long long)L.S * L.Tmax, L.Fs, kBNs[i]);
   }
+  if (ok && !L.w8) ok = encode_2d(&m->xperm, xperm, rows, L.d, kPairRows);
   if (!ok) {
     delete m;
     if (msg) *msg = "cuTensorMapEncodeTiled rejected a weight or workspace tensor";
@@ -1883,22 +1888,19 @@ cudaError_t tc_launch_up(const TcLayer& L, const TcCall& c, bool shared, cudaStr
     if (m->il4 && m->sil4) {
       a.gate_first = m->gate_first ? 1 : 0;
       sa.gate_first = m->sgate_first ? 1 : 0;
-      return launch_pair<kModeGateUpIL, true>(L, one_kb, m->wgu4, m->wgu4,
-                                              m->xperm[bn_index(kPairRows)], a, units + s_units,
-                                              st, &m->wsgu4, &m->wsgu4, &xm, &sa);
+      return launch_pair<kModeGateUpIL, true>(L, one_kb, m->wgu4, m->wgu4, m->xperm, a,
+                                              units + s_units, st, &m->wsgu4, &m->wsgu4, &xm, &sa);
     }
-    return launch_pair<kModeGateUpIL>(L, one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
-                                      units + s_units, st, &m->wsg64, &m->wsu64, &xm, &sa);
+    return launch_pair<kModeGateUpIL>(L, one_kb, m->wg64, m->wu64, m->xperm, a, units + s_units, st,
+                                      &m->wsg64, &m->wsu64, &xm, &sa);
   }
   if (pair && m->il4) {
     a.gate_first = m->gate_first ? 1 : 0;
-    return launch_pair<kModeGateUpIL, true>(L, one_kb, m->wgu4, m->wgu4,
-                                            m->xperm[bn_index(kPairRows)], a, units, st);
+    return launch_pair<kModeGateUpIL, true>(L, one_kb, m->wgu4, m->wgu4, m->xperm, a, units, st);
   }
   if (pair)
-    return launch_pair<kModeGateUpIL>(L, one_kb, m->wg64, m->wu64, m->xperm[bn_index(kPairRows)], a,
-                                      units, st);
-  return up_bn(m->wg, m->wu, L.w8 ? m->xq[bn_index(bn)] : m->xperm[bn_index(bn)], grid);
+    return launch_pair<kModeGateUpIL>(L, one_kb, m->wg64, m->wu64, m->xperm, a, units, st);
+  return up_bn(m->wg, m->wu, L.w8 ? m->xq[bn_index(bn)] : m->xperm, grid);
 }
 
 cudaError_t tc_launch_down(const TcLayer& L, const TcCall& c, bool shared, int n_split,
