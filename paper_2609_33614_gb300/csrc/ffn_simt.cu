@@ -12,12 +12,19 @@
 //
 // What bounds it: a large call the shared-memory reads (8 x 8 outputs per thread need one 16-byte
 // read per 16 FMAs), a small call the latency of one block's tile lookup, copies and sums.  Hence
-// three shapes, by the call's (selected rows) x (expert width); the layer of 8 experts, width 512
-// and d_model 256 measured, us per forward call (small / mid / large shape):
-//   tokens      64    128    384    512    768   1536   1999   3000   4096
-//   small     27.7   34.4   71.4   80.8  106.2  174.8  214.1  303.7  404.2
-//   mid       40.2   46.6   76.2   81.3   93.5  123.5  158.0  203.8  268.7
-//   large     62.1   63.3   91.7  103.8  117.6  146.2  155.6  193.3  266.7
+// three shapes, by the call's (selected rows) x (expert width); the layer of 8 experts, K = 2, width
+// 512 and d_model 256, us per forward call in a graph (small / mid / large shape):
+//   tokens   64   128   384   512   768  1300  1536  1850  1999  2200  3000  4096
+//   small  25.7  33.5  55.0  64.7  90.5 137.1 157.7 189.1 200.0 218.8 286.9 382.8
+//   mid    35.8  41.2  58.0  64.2  77.2  95.5 106.5 135.7 144.6 150.3 186.3 248.4
+//   large  57.9  59.1  73.4  96.1 100.3 122.4 135.6 141.5 141.9 142.4 177.1 246.4
+// The line between small and mid lies there for the other layers measured too (64 experts, K = 8,
+// width 1024, d 2048: 64 tokens 389 / 382; 16 experts, K = 2, width 1024, d 512: 200 85 / 84, 300 116 /
+// 118; 8 experts, width 2048, d 2048: 64 202 / 261, 128 345 / 314).  Mid and large cross at 200 to 500
+// rows per expert, which the toy layer reaches at its line (1953 tokens) and wider layers later than
+// theirs: the layer of 64 experts mid / large 300 tokens 1107 / 1298, 1300 3723 / 3784, 1536 4311 /
+// 4232; that of 16 experts 1300 273 / 300, 1536 312 / 303, 1999 406 / 430, 3000 574 / 568; 8 experts of
+// width 2048 512 806 / 1026, 1000 1436 / 1456, 2200 2911 / 2803.
 // (the kernels before, 32 x 64 tiles with 2 x 4 outputs per thread and one chunk in flight: gate/up
 // and down 26.6 + 46.1 us at 64 tokens, 108 + 95 us at 1999.)
 #include "eat_internal.cuh"
@@ -290,7 +297,7 @@ cudaError_t simt_configure() {
 }
 
 SimtShape simt_shape(int T, int K, int F) {
-  // selected rows x width: the lines of the table at the top of this file (512 and 1999 tokens)
+  // selected rows x width: where the columns of the table at the top of this file cross
   const long long work = (long long)T * K * F;
   return work >= 2000000 ? SimtShape::kLarge
                          : work >= 512 * 1024 ? SimtShape::kMid : SimtShape::kSmall;

@@ -15,9 +15,10 @@
 //       it, bf16 rows O[slot][c].
 // Persistent CTAs (one per SM) walk the work units (token tile, feature tile, K slice) of all
 // groups; the group sizes live on the device (written by the permute kernel), so no host sync.
-// Warp roles: warp 0 lane 0 issues TMA; warp 1 owns TMEM and lane 0 issues MMAs; warps 2-5 (and
-// 6-9 for e4m3 tiles of 64 or more tokens, each warp half of the tile's columns) drain TMEM
-// (double-buffered accumulators, so the epilogue of tile i overlaps the MMAs of tile i + 1).
+// Warp roles: one elected lane of warp 0 issues TMA; warp 1 owns TMEM and one elected lane of it
+// issues MMAs; warps 2-5 (and 6-9 for e4m3 tiles of 64 or more tokens, each warp half of the tile's
+// columns) drain TMEM (double-buffered accumulators, so the epilogue of tile i overlaps the MMAs of
+// tile i + 1).
 // Every mbarrier wait is bounded (2 s); on expiry the kernel records an error in the device status
 // word, lets in-flight copies and MMAs finish, frees its TMEM and returns.
 #include "ffn_tc.cuh"
@@ -257,8 +258,8 @@ struct Cfg {
                               : 6 * kSubBytes <= kSmemBudget - 2048                          ? 2
                                                                                              : 1;
   // e4m3 tiles of 64 or more tokens are drained by two warps per TMEM lane quarter (one per half
-  // of the tile's columns), so an accumulator buffer returns to the MMA issuer sooner (e4m3
-  // prefill +20 %)
+  // of the tile's columns), so an accumulator buffer returns to the MMA issuer sooner (e4m3 calls of
+  // 4096 tokens, which now run on SM pairs, were 20 % faster with eight)
   static constexpr int kEpiWarps = (W8 && BN >= 64) ? 8 : 4;
   static constexpr int kThreads = 64 + 32 * kEpiWarps;
   static constexpr int kStageBytes = kKPS * kSubBytes;
@@ -720,8 +721,8 @@ tc_ffn_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__
 // ------------------------------------------------------------ SM-pair kernels (cta_group::2)
 // Large calls run on pairs of SMs (2-CTA clusters).  The pair issues M = 256 x N = 256 MMAs: each
 // CTA holds 128 rows of A (weight rows) and 128 of the tile's 256 token rows of B, so a k-block is
-// 32 KB per SM for the flops the single-SM kernel stages in 48 KB; a pipeline stage holds two
-// k-blocks and three stages are in flight.  Rank 0 of the pair
+// 32 KB per SM for the flops the single-SM kernel stages in 48 KB; three stages of two k-blocks are
+// in flight, or seven of one (PairCfg).  Rank 0 of the pair
 // issues the MMAs (tcgen05.mma.cta_group::2) and commits them to the barriers of both CTAs; both
 // CTAs load their halves with TMA completing on rank 0's full barrier (rank 0 expects the bytes
 // of both); each CTA drains its own TMEM rows, and rank 0 reuses an accumulator buffer once the
@@ -1557,18 +1558,22 @@ cudaError_t configure_kernels(TcLayer& L) {
 // least kPairMinTokens tokens, or with kPairMinRows per expert on average, run both expert GEMMs on
 // SM pairs with 256-token tiles (interleaved gate/up, 256-feature down tiles); smaller calls use
 // single-SM kernels with tiles of the smallest width that holds T, at most 128.  us per call, single
-// SM / pairs: Mixtral shape 200 tokens (50 rows per expert) 482 / 476, 400 618 / 536, 1000 978 /
-// 785; OLMoE 333 (41) 131 / 151, 600 (75) 159 / 159, 1000 205 / 194; Qwen 600 (40) 192 / 177, 1000
-// 234 / 203; DeepSeek-V2-Lite 333 (31) 209 / 223, 600 (56) 231 / 233, 1000 300 / 265.  (On a single
-// SM the interleaved 256-token gate/up moves the same shared-memory bytes per flop as two 128-token
-// accumulators and measured slower: OLMoE prefill gate/up 294 -> 316 us.)
+// SM / pairs: Mixtral shape 257 tokens (64 rows per expert) 476 / 474, 300 565 / 478, 1000 911 / 692;
+// OLMoE 333 (42) 132 / 151, 400 (50) 136 / 139, 450 (56) 144 / 140, 512 (64) 154 / 144, 1000 196 /
+// 188; DeepSeek-V2-Lite 333 (31) 213 / 223, 450 (42) 219 / 233, 500 226 / 224, 600 242 / 231, 1000
+// 304 / 262; 128 experts of K = 8 (d 2048, F 768) 450 (28) 132 / 133, 512 134 / 137, 600 141 / 139, 700
+// 147 / 151, 800 164 / 163; Qwen 512 (34) 175 / 152.  (On a single SM the interleaved 256-token
+// gate/up moves the same shared-memory bytes per flop as two 128-token accumulators and measured
+// slower: OLMoE prefill gate/up 294 -> 316 us.)
 //   So do calls of more than 128 tokens whose shared experts would have too many 128-token units to
-// run beside the routing: on pairs they either have few enough again or follow the routed units in the
-// same launches, where the single-SM kernels give them launches of their own.  Single SM / pairs:
-// Qwen 385 tokens 172 / 142, 450 179 / 150, 511 176 / 160; with shared experts twice as wide 129
-// 139 / 111, 257 163 / 149, 384 187 / 164; one shared expert of 8192 features (128 experts, K = 1) 257
-// 129 / 95.  64 experts with K = 8 and two shared experts of 5632 lose in a part of their range: 200
-// 184 / 166, 333 202 / 217, 500 232 / 207.
+// run beside the routing: on pairs they either have few enough again or follow the routed units in
+// the same launches, where the single-SM kernels give them launches of their own.  Single SM / pairs:
+// Qwen 385 tokens 173 / 140, 511 175 / 152; with shared experts twice as wide 129 138 / 112, 257 172 /
+// 152, 384 186 / 170; one shared expert of 8192 features (128 experts, K = 1) 257 129 / 93; one of
+// 16384 (32 experts, K = 4) 129 193 / 127, 257 221 / 209.  64 experts with a large K lose in a part of
+// the range, where the routed units lose more on pairs than the shared ones gain: K = 8 and two shared
+// experts of 5632, 200 184 / 162, 257 193 / 199, 333 215 / 219, 384 217 / 195; K = 6 and one of 11264,
+// 256 189 / 154, 333 206 / 217, 384 209 / 214, 450 223 / 220.
 constexpr int kPairMinTokens = 512, kPairMinRows = 64;
 bool tc_shared_beside(const TcLayer& L, int T, int tile_rows) {
   const long long units =
@@ -1601,11 +1606,14 @@ static int streams_weights(int T) { return T <= kBNs[kNumBN - 1] ? 1 : 0; }
 // 174.0.
 static bool pairs8(const TcLayer& L, int T) { return L.w8 && T > kBNs[kNumBN - 1]; }
 
-// bf16 SM pairs: one k-block per stage for calls of at most 512 rows per expert on average.  us per
-// call, two / one: OLMoE 600 tokens 158.8 / 154.6, 4096 (512 rows) 410.8 / 403.8, 10000 (1250) 861 /
-// 868; Mixtral shape 400 534 / 514, 2000 (500) 1236 / 1183; DeepSeek-V2-Lite 1500 309 / 296, 4096
-// (384) 516 / 511, 16384 (1536) 1685 / 1692; Qwen 1000 202 / 197, 8192 (546, beside shared experts'
-// full tiles) 844 / 871.
+// bf16 SM pairs: one k-block per stage for calls of at most 512 rows per expert on average: it gains up
+// to about 400 rows, and from there on neither does.  us per call, two / one: Mixtral shape 1024
+// tokens (256 rows) 713 / 677, 1500 (375) 991 / 963, 2048 (512) 1216 / 1229, 4096 (1024) 2307 / 2268;
+// OLMoE 2048 (256) 270 / 267, 3000 (375) 345 / 341, 4096 (512) 424 / 424, 5000 (625) 488 / 497, 7000
+// (875) 661 / 652, 12000 (1500) 1055 / 1079; DeepSeek-V2-Lite 2048 (192) 353 / 346, 4096 (384) 539 /
+// 534, 6000 (562) 728 / 735, 12000 (1125) 1337 / 1343; 32 experts, K = 4, d 4096: 2048 (256) 493 / 479,
+// 4096 (512) 754 / 754, 6000 (750) 1025 / 1031; Qwen 2048 (137) 310 / 306, 4096 (273) 497 / 504, 8192
+// (546) 926 / 931.
 static bool pair_one_kb(const TcLayer& L, int T) {
   return (long long)T * L.K <= 512LL * L.E;
 }

@@ -142,8 +142,7 @@ __device__ __forceinline__ void store_x4(__nv_bfloat16* p, const X4b& v) { *(uin
 // xcopy (or null): x is read from memory the caller keeps on the host (a host-buffer call) and
 // warp 0 of the blocks of the first expert group also writes what it reads to xcopy, the device
 // copy every later kernel of the call reads.
-// (bf16 x: at most 32 registers, so eight blocks share an SM and a 32-token decode call of a
-// 64-expert layer, 1024 blocks, runs in one wave)
+// (bf16 x: at most 32 registers, so eight blocks share an SM: each is short and waits for its loads)
 template <typename TX>
 __global__ void __launch_bounds__(kLogitThreads, sizeof(TX) == 2 ? 8 : 1)
 router_logits_small_kernel(const TX* __restrict__ x, const float* __restrict__ wr, int T, int d,
@@ -821,7 +820,8 @@ route_select_kernel(const float2* __restrict__ part, int n_split, const SelectAr
 // registers are bounded so that three CTAs share an SM (a second wave of clusters of eight took
 // 9.1 us instead of 5.6 at 16 tokens).  us per routing call (graph of 10), two kernels / this one:
 // OLMoE 32 tokens 7.0 / 6.2, 128 12.3 / 8.1, 1 5.4 / 6.0; Mixtral 1 6.4 / 4.6, 64 7.5 / 6.0, 300
-// 20.3 / 13.5; the fp32 toy layer 64 5.8 / 4.7.
+// 20.3 / 13.5; the fp32 toy layer 64 5.8 / 4.7.  The register bounds (72 up to 32 experts, 96 above)
+// cost TT = 4 124-128 and 28-48 bytes of spills.
 constexpr int kFusedSlice = 512;
 constexpr int kFusedMaxSlices = 8;  // portable cluster size
 // Warps that compute scores: 16 take the 64 experts of one token in one round.

@@ -2,7 +2,7 @@
 
 Argument marshalling only: every step of the layer runs in the CUDA library.  torch tensors are
 used for device memory and streams; pointers are passed as ``tensor.data_ptr()`` and the stream
-as ``torch.cuda.current_stream().cuda_stream``.  Loading fails loudly when the library is missing:
+as the handle of torch's current stream (``_stream``).  Loading fails loudly when the library is missing:
 there is no CPU fallback.
 """
 from __future__ import annotations
